@@ -262,18 +262,6 @@ bool overlap(const hom_inclusion& p, const hom_inclusion& q, const double* Y, in
   return std::sqrt(s) < bl.size[0];
 }
 
-void make_plan(int M, FftPlan& p) {
-  p.M = M;
-  p.nrad = 0;
-  p.sched = 0;
-  int m = M;
-  const int small[] = {5, 3, 7, 11, 13, 2};   // 2 only for image lengths (the double grid is odd)
-  for (int r : small)
-    while (m % r == 0 && p.nrad < kMaxRadices) { p.radix[p.nrad++] = r; m /= r; }
-  for (int r = 17; m > 1 && r <= m; r += 2)
-    while (m % r == 0 && p.nrad < kMaxRadices) { p.radix[p.nrad++] = r; m /= r; }
-}
-
 // Smallest odd M >= m whose prime factors are all radices with butterflies (3, 5, 7, 11,
 // 13). The double-grid quadrature (Lemma double-grid) stays exact on any odd M >= 2N - 1:
 // the Galerkin entries need A_hat(k - j) for |k - j| <= N - 1, all inside Z_M without
@@ -1523,8 +1511,8 @@ hom_status build_batch(hom_ctx* ctx, int n, const hom_problem* probs, const hom_
       pack_sym(side == 0 ? A0f : B0, 2, g.ncomp, t.C0p);
       t.tw0 = tw_off(g.M[0]);
       t.tw1 = tw_off(g.M[1]);
-      t.plan0 = g.plan[0];
-      t.plan1 = g.plan[1];
+      make_plan(g.M[0], t.plan0, false);
+      make_plan(g.M[1], t.plan1, false);
       for (size_t j = 0; j < g.incl.size(); ++j) {
         const hom_inclusion& I = g.incl[j];
         DevIncl D;

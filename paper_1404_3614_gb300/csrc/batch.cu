@@ -73,7 +73,7 @@ __device__ __noinline__ cpx<T>* fft_sched(cpx<T>* a, cpx<T>* b, int G, int M, co
     case 125: return cfft_from<T, 125, 0, BIG>(a, b, G, W, dir);
     case 225: return cfft_from<T, 225, 0, BIG>(a, b, G, W, dir);
     case 405: return cfft_from<T, 405, 0, BIG>(a, b, G, W, dir);
-    default: return fft_pencils<T>(a, b, G, M, plan, W, dir);
+    default: return fft_pencils_small<T>(a, b, G, M, plan, W, dir);
   }
 }
 

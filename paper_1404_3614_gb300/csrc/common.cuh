@@ -96,14 +96,74 @@ __host__ __device__ constexpr int cf_ns(int M, int stage, bool big = false) {
   return p;
 }
 
-// Factorised plan of one odd transform length M (Stockham autosort, mixed radix).
+// FastDiv's multiplier and shift alone (an aggregate: all zero until set).
+struct DivConst {
+  uint32_t m, s;
+};
+__host__ __device__ inline DivConst div_const(uint32_t d) {
+  const FastDiv f(d);
+  return DivConst{f.m, f.s};
+}
+__device__ __forceinline__ int div_by(DivConst c, int n) { return (int)((__umulhi((uint32_t)n, c.m) + (uint32_t)n) >> c.s); }
+
+// Factorised plan of one transform length M (Stockham autosort, mixed radix). Inverse
+// transforms run the radices in order, forward ones in reverse order, so that the stage with
+// the most to skip (the largest radix) is the first of a zero-padded inverse transform and the
+// last of a truncating forward one.
+constexpr int kPlanDivs = 8;
 struct FftPlan {
   int M;
   int nrad;
   int radix[kMaxRadices];
   int sched;   // compile-time lengths in the batched kernel: 0 precision default,
                // 1 radices 5 and 3, 2 composite register radices 15, 25, 9
+  int ndiv;    // > 0: the divisions of a stage prepared (plan_divisions), else formed in the kernel
+  DivConst nb[kPlanDivs];   // by M / radix[s]
+  DivConst nsi[kPlanDivs];  // by the product of the radices before s (inverse order)
+  DivConst nsf[kPlanDivs];  // by the product of the radices after s (forward order)
 };
+__host__ __device__ inline void plan_divisions(FftPlan& p) {
+  p.ndiv = 0;
+  if (p.nrad > kPlanDivs) return;
+  int ns = 1;
+  for (int s = 0; s < p.nrad; ++s) {
+    p.nb[s] = div_const((uint32_t)(p.M / p.radix[s]));
+    p.nsi[s] = div_const((uint32_t)ns);
+    ns *= p.radix[s];
+  }
+  ns = 1;
+  for (int s = p.nrad - 1; s >= 0; --s) {
+    p.nsf[s] = div_const((uint32_t)ns);
+    ns *= p.radix[s];
+  }
+  p.ndiv = p.nrad;
+}
+
+// Radices of a transform of length M: primes above 13 first (their first inverse stage skips
+// the zero padding's terms and needs no twiddles), then with `big` the composite register
+// radices 15 and 9 (fewer passes through shared memory), then 13, 11, 7, 5, 3 and, for image
+// lengths and even grids (the double grid is odd), 8, 4, 2. The batched kernel takes radices
+// 5, 3, 7, 11, 13 in this order (big = false, see fft_pencils_small).
+inline void make_plan(int M, FftPlan& p, bool big = true) {
+  p.M = M;
+  p.nrad = 0;
+  p.sched = 0;
+  int rest[kMaxRadices], nrest = 0;
+  auto pull = [&](int& m, int r) {
+    while (m % r == 0 && nrest < kMaxRadices) { rest[nrest++] = r; m /= r; }
+  };
+  int m = M;
+  if (big)
+    for (int r : {15, 13, 11, 9, 7, 5, 3, 8, 4, 2}) pull(m, r);
+  else
+    for (int r : {5, 3, 7, 11, 13}) pull(m, r);
+  for (int r = 17; m > 1; r += 2) {
+    if ((long long)r * r > m) r = m;   // what is left is prime
+    while (m % r == 0 && p.nrad < kMaxRadices) { p.radix[p.nrad++] = r; m /= r; }
+  }
+  for (int i = 0; i < nrest && p.nrad < kMaxRadices; ++i) p.radix[p.nrad++] = rest[i];
+  plan_divisions(p);
+}
 
 // ---------------------------------------------------------------------------------
 // Small DFT butterflies. dir = -1: forward (w = exp(-2 pi i / r)); dir = +1: inverse.
@@ -410,9 +470,342 @@ __device__ __forceinline__ void dft15_zout(cpx<T>* v, int dir) {
   v[14] = b[4];
 }
 
-// Generic compile-time radix R from registers, roots from the length-M table W.
+// Inputs a zero-padded inverse transform of N <= (M + 1) / 2 frequencies knows to be zero in
+// a first stage of odd radix R, and outputs a truncating forward one drops in a last stage:
+// q = LO .. R - 1 - LO (positions q M / R + j around the middle of the pencil).
+template <int R> struct RadixBand {
+  static constexpr int lo = R / 4 + 1, hi = R - 1 - lo;
+  static constexpr bool in(int q) { return q >= lo && q <= hi; }
+};
+// whether those positions hold nothing when the frequencies 0 .. half and -top .. -1 are stored
+__device__ __forceinline__ bool radix_band_free(int R, int nb, int M, int half, int top) {
+  const int lo = R / 4 + 1;
+  return lo * nb > half && (R - lo) * nb <= M - top;
+}
+
+// Odd radix R in registers from the sums a_q = v_q + v_{R-q} and differences b_q = v_q - v_{R-q}
+// (DFT of a_q with cosines, of b_q with sines: a quarter of the products of the direct sum):
+// V_s, V_{R-s} = v_0 + sum_q a_q cos(2 pi q s / R) +- i DIR sum_q b_q sin(2 pi q s / R).
+// ZI: the inputs of RadixBand are zero (not read); ZO: its outputs are not needed (undefined).
+template <typename T, int R, int DIR, bool ZI = false, bool ZO = false>
+__device__ __forceinline__ void dft_odd(cpx<T>* v) {
+  constexpr int H = (R - 1) / 2, LO = RadixBand<R>::lo;
+  constexpr int QN = ZI ? (LO < H ? LO : H) : H;   // pairs with a nonzero input
+  constexpr int SN = ZO ? (LO < H ? LO : H) : H;   // pairs with a needed output
+  cpx<T> a[QN], b[QN];
+#pragma unroll
+  for (int q = 1; q <= QN; ++q) {
+    if (ZI && RadixBand<R>::in(q)) {   // only v_{R-q}
+      a[q - 1] = v[R - q];
+      b[q - 1] = mk<T>(-v[R - q].x, -v[R - q].y);
+    } else {
+      a[q - 1] = add<T>(v[q], v[R - q]);
+      b[q - 1] = sub<T>(v[q], v[R - q]);
+    }
+  }
+  const cpx<T> v0 = v[0];
+  cpx<T> t0 = v0;
+#pragma unroll
+  for (int q = 0; q < QN; ++q) t0 = add<T>(t0, a[q]);
+  v[0] = t0;
+#pragma unroll
+  for (int s = 1; s <= SN; ++s) {
+    cpx<T> m = v0, n;
+#pragma unroll
+    for (int q = 1; q <= QN; ++q) {
+      const T c = T(ct_cos2pi(q * s, R)), sn = T(DIR * ct_sin2pi(q * s, R));
+      m = mk<T>(fma(c, a[q - 1].x, m.x), fma(c, a[q - 1].y, m.y));
+      if (q == 1) n = mk<T>(sn * b[0].x, sn * b[0].y);
+      else n = mk<T>(fma(sn, b[q - 1].x, n.x), fma(sn, b[q - 1].y, n.y));
+    }
+    if (!(ZO && RadixBand<R>::in(s))) v[s] = mk<T>(m.x - n.y, m.y + n.x);
+    v[R - s] = mk<T>(m.x + n.y, m.y - n.x);
+  }
+}
+
+// Radix 9 = 3 x 3 with its middle inputs 3..5 zero (ZI) or its middle outputs 3..5 not needed (ZO)
+template <typename T> __device__ __forceinline__ void dft3_mid_in0(cpx<T>* v, int dir);
+template <typename T> __device__ __forceinline__ void dft3_skip_out1(cpx<T>* v, int dir);
+template <typename T, int DIR, bool ZI, bool ZO>
+__device__ __forceinline__ void dft9_band(cpx<T>* v) {
+  cpx<T> t[9];
+#pragma unroll
+  for (int n2 = 0; n2 < 3; ++n2) {
+    cpx<T> a[3] = {v[n2], v[3 + n2], v[6 + n2]};
+    if (ZI) dft3_mid_in0<T>(a, DIR);
+    else dft3<T>(a, DIR);
+#pragma unroll
+    for (int k1 = 0; k1 < 3; ++k1) {
+      if (n2 * k1 == 0) {
+        t[n2 * 3 + k1] = a[k1];
+      } else {
+        const T c = T(ct_cos2pi(n2 * k1, 9)), s = T(DIR * ct_sin2pi(n2 * k1, 9));
+        t[n2 * 3 + k1] = mk<T>(fma(a[k1].x, c, -a[k1].y * s), fma(a[k1].x, s, a[k1].y * c));
+      }
+    }
+  }
+#pragma unroll
+  for (int k1 = 0; k1 < 3; ++k1) {
+    cpx<T> b[3] = {t[k1], t[3 + k1], t[6 + k1]};
+    if (ZO) dft3_skip_out1<T>(b, DIR);
+    else dft3<T>(b, DIR);
+    v[k1] = b[0];
+    if (!ZO) v[3 + k1] = b[1];
+    v[6 + k1] = b[2];
+  }
+}
+
+// Power-of-two radices 2, 4, 8 (image lengths and even grids; the double grid is odd)
+template <typename T, int R, int DIR>
+__device__ __forceinline__ void dft_pow2(cpx<T>* v) {
+  if constexpr (R == 2) {
+    const cpx<T> a = v[0];
+    v[0] = add<T>(a, v[1]);
+    v[1] = sub<T>(a, v[1]);
+  } else {
+    constexpr int Hh = R / 2;
+    cpx<T> e[Hh], o[Hh];
+#pragma unroll
+    for (int k = 0; k < Hh; ++k) {
+      e[k] = v[2 * k];
+      o[k] = v[2 * k + 1];
+    }
+    dft_pow2<T, Hh, DIR>(e);
+    dft_pow2<T, Hh, DIR>(o);
+#pragma unroll
+    for (int k = 0; k < Hh; ++k) {
+      cpx<T> w = o[k];
+      if (4 * k == R) {
+        w = rot<T>(w, DIR);
+      } else if (k > 0) {
+        const T c = T(ct_cos2pi(k, R)), s = T(DIR * ct_sin2pi(k, R));
+        w = mk<T>(fma(o[k].x, c, -o[k].y * s), fma(o[k].x, s, o[k].y * c));
+      }
+      v[k] = add<T>(e[k], w);
+      v[k + Hh] = sub<T>(e[k], w);
+    }
+  }
+}
+
+template <typename T, int R, int DIR, bool ZI, bool ZO>
+__device__ __forceinline__ void dft_radix(cpx<T>* v) {
+  if constexpr (R % 2 == 0) dft_pow2<T, R, DIR>(v);
+  else if constexpr (R == 3 && ZI) dft3_mid_in0<T>(v, DIR);
+  else if constexpr (R == 3 && ZO) dft3_skip_out1<T>(v, DIR);
+  else if constexpr (R == 3) dft3<T>(v, DIR);
+  else if constexpr (R == 9) dft9_band<T, DIR, ZI, ZO>(v);
+  else if constexpr (R == 15 && ZI) dft15_zin<T>(v, DIR);
+  else if constexpr (R == 15 && ZO) dft15_zout<T>(v, DIR);
+  else if constexpr (R == 15) dft15_pfa<T>(v, DIR);
+  else if constexpr (R == 5 && !ZI && !ZO) dft5<T>(v, DIR);
+  else dft_odd<T, R, DIR, ZI, ZO>(v);
+}
+
+// One Stockham stage of radix R over G pencils (strides ld) of runtime length M.
+template <typename T, int R, int DIR, bool ZI, bool ZO>
+__device__ __forceinline__ void stage_radix(const cpx<T>* __restrict__ a, cpx<T>* __restrict__ b, int G, int ld, int M,
+                                            int Ns, DivConst dnb, DivConst dns, const cpx<T>* W) {
+  const int nb = M / R;
+  const int step = nb / Ns;   // M / (Ns R)
+  for (int t = threadIdx.x; t < G * nb; t += blockDim.x) {
+    const int g = div_by(dnb, t);
+    const int j = t - g * nb;
+    const cpx<T>* src = a + (size_t)g * ld + j;
+    cpx<T> v[R];
+#pragma unroll
+    for (int q = 0; q < R; ++q)
+      if (!(ZI && RadixBand<R>::in(q))) v[q] = src[q * nb];
+    int base = j * R;
+    if (Ns > 1) {
+      const int c = div_by(dns, j);
+      const int k = j - c * Ns;
+      base = c * Ns * R + k;
+      const int kw = k * step;
+#pragma unroll
+      for (int q = 1; q < R; ++q) v[q] = mulc<T>(v[q], W[q * kw], DIR > 0);
+    }
+    dft_radix<T, R, DIR, ZI, ZO>(v);
+    cpx<T>* dst = b + (size_t)g * ld + base;
+#pragma unroll
+    for (int q = 0; q < R; ++q)
+      if (!(ZO && RadixBand<R>::in(q))) dst[q * Ns] = st_norm<T>(v[q]);
+  }
+}
+
+// A stage of any larger prime radix R (twice: the callers synchronise in between). First the
+// twiddled inputs' sums x_q + x_{R-q} and differences x_q - x_{R-q}, in place at q and R - q;
+// then each thread forms kPrimeTile output pairs (s, R - s) of one butterfly from them:
+// R / 2 terms of two real products a complex output instead of R terms of eight, one load of a
+// sum and a difference for kPrimeTile pairs. qn, sn: pairs with a nonzero input / a needed output.
+constexpr int kPrimeTile = 4;
+template <typename T, int DIR>
+__device__ __forceinline__ void stage_prime_sums(cpx<T>* a, int G, int ld, int M, int R, int Ns, int qn,
+                                                 DivConst dnb, DivConst dns, const cpx<T>* W) {
+  const int nb = M / R;
+  const int step = nb / Ns;
+  for (int t = threadIdx.x; t < G * nb * qn; t += blockDim.x) {
+    const int gj = t / qn;
+    const int q = t - gj * qn + 1;
+    const int g = div_by(dnb, gj);
+    const int j = gj - g * nb;
+    cpx<T>* p = a + (size_t)g * ld + j;
+    cpx<T> x = p[q * nb], y = p[(R - q) * nb];
+    if (Ns > 1) {
+      const int k = j - div_by(dns, j) * Ns;
+      x = mulc<T>(x, W[q * k * step], DIR > 0);
+      y = mulc<T>(y, W[(R - q) * k * step], DIR > 0);
+    }
+    p[q * nb] = st_norm<T>(add<T>(x, y));
+    p[(R - q) * nb] = st_norm<T>(sub<T>(x, y));
+  }
+}
+template <typename T, int DIR>
+__device__ __forceinline__ void stage_prime_out(const cpx<T>* __restrict__ a, cpx<T>* __restrict__ b, int G, int ld,
+                                                int M, int R, int Ns, int qn, int sn, DivConst dnb, DivConst dns,
+                                                const cpx<T>* W) {
+  const int nb = M / R;
+  const int ntile = (sn + kPrimeTile) / kPrimeTile;   // s = 0 .. sn
+  const int nbf = G * nb;
+  for (int t = threadIdx.x; t < nbf * ntile; t += blockDim.x) {
+    const int tile = t / nbf;
+    const int gj = t - tile * nbf;
+    const int g = div_by(dnb, gj);
+    const int j = gj - g * nb;
+    const cpx<T>* p = a + (size_t)g * ld + j;
+    const int s0 = tile * kPrimeTile;
+    const cpx<T> x0 = p[0];
+    cpx<T> m[kPrimeTile], n[kPrimeTile];
+    int ws[kPrimeTile];
+#pragma unroll
+    for (int u = 0; u < kPrimeTile; ++u) {
+      m[u] = x0;
+      n[u] = mk<T>(T(0), T(0));
+      ws[u] = 0;
+    }
+    for (int q = 1; q <= qn; ++q) {
+      const cpx<T> sa = p[q * nb], sb = p[(R - q) * nb];
+#pragma unroll
+      for (int u = 0; u < kPrimeTile; ++u) {
+        ws[u] += s0 + u;
+        if (ws[u] >= R) ws[u] -= R;
+        const cpx<T> w = W[ws[u] * nb];   // cos, -sin of 2 pi q s / R
+        m[u] = mk<T>(fma(w.x, sa.x, m[u].x), fma(w.x, sa.y, m[u].y));
+        n[u] = mk<T>(fma(w.y, sb.x, n[u].x), fma(w.y, sb.y, n[u].y));
+      }
+    }
+    const int c = div_by(dns, j);
+    const int k = j - c * Ns;
+    cpx<T>* d = b + (size_t)g * ld + c * Ns * R + k;
+#pragma unroll
+    for (int u = 0; u < kPrimeTile; ++u) {
+      const int s = s0 + u;
+      if (s > sn || 2 * s >= R) continue;
+      // n holds - sum b sin: V_s = m + i DIR sum b sin
+      const cpx<T> in = DIR > 0 ? mk<T>(n[u].y, -n[u].x) : mk<T>(-n[u].y, n[u].x);
+      d[s * Ns] = st_norm<T>(add<T>(m[u], in));
+      if (s > 0) d[(R - s) * Ns] = st_norm<T>(sub<T>(m[u], in));
+    }
+  }
+}
+
+// The frequencies around 0 that a pencil holds (0 .. half and -top .. -1) and which side of the
+// transform they bound: prune bit 1, zero-padded inputs (the first stage skips its known
+// zeros); bit 2, truncated outputs (the last stage skips what is dropped).
+struct FftBand {
+  int half, top, prune;
+};
+
+// the pairs (q, R - q), q <= h, of rows of `stride` positions with one inside the band
+__device__ __forceinline__ int pairs_in_band(int h, int stride, FftBand band) {
+  const int up = band.half / stride, dn = (band.top + stride - 1) / stride;
+  const int n = up > dn ? up : dn;
+  return n < h ? n : h;
+}
+
+// G pencils of length M at a + g*ld (ping-pong with b, same strides) by the runtime plan, in
+// direction DIR. The CTA runs all stages; returns the buffer holding the result. Ends with
+// __syncthreads().
+// Bound by instruction issue (FP32, float-float) or the FP64 pipe: so the index divisions by
+// runtime lengths are multiplications prepared in the plan, radices 15 and 9 halve the passes
+// through shared memory, radices 5 to 13 and primes use the real symmetry, and zero padding and
+// dropped outputs are skipped. Against radices 3, 5, 7 with divisions and direct sums: FP32
+// operator of a 41 x 33 x 53 cell (lengths 81, 65, 105) 298 -> 92 us, mixed bounds of 16 balls at
+// N = 51 (length 105) 176 -> 72 ms, FP64 3D operators at lengths with primes 4 to 7 times.
+template <typename T, int DIR>
+__device__ __forceinline__ cpx<T>* fft_plan_run(cpx<T>* a, cpx<T>* b, int G, int ld, const FftPlan& plan,
+                                                const cpx<T>* W, FftBand band) {
+  const int M = plan.M;
+  int Ns = 1;
+  cpx<T>* src = a;
+  cpx<T>* dst = b;
+  for (int i = 0; i < plan.nrad; ++i) {
+    const int s = DIR > 0 ? i : plan.nrad - 1 - i;
+    const int R = plan.radix[s];
+    const int nb = M / R;
+    DivConst dnb, dns;
+    if (plan.ndiv > 0) {
+      dnb = plan.nb[s];
+      dns = DIR > 0 ? plan.nsi[s] : plan.nsf[s];
+    } else {
+      dnb = div_const((uint32_t)nb);
+      dns = div_const((uint32_t)Ns);
+    }
+    const bool free_ = radix_band_free(R, nb, M, band.half, band.top);
+    const bool zi = DIR > 0 && (band.prune & 1) && i == 0 && free_;
+    const bool zo = DIR < 0 && (band.prune & 2) && i == plan.nrad - 1 && free_;
+#define HOMB_STAGE(RR)                                                                                        \
+  case RR:                                                                                                    \
+    if (DIR > 0 && zi) stage_radix<T, RR, DIR, (DIR > 0), false>(src, dst, G, ld, M, Ns, dnb, dns, W);        \
+    else if (DIR < 0 && zo) stage_radix<T, RR, DIR, false, (DIR < 0)>(src, dst, G, ld, M, Ns, dnb, dns, W);   \
+    else stage_radix<T, RR, DIR, false, false>(src, dst, G, ld, M, Ns, dnb, dns, W);                          \
+    break;
+    switch (R) {
+      case 2: stage_radix<T, 2, DIR, false, false>(src, dst, G, ld, M, Ns, dnb, dns, W); break;
+      case 4: stage_radix<T, 4, DIR, false, false>(src, dst, G, ld, M, Ns, dnb, dns, W); break;
+      case 8: stage_radix<T, 8, DIR, false, false>(src, dst, G, ld, M, Ns, dnb, dns, W); break;
+      HOMB_STAGE(3)
+      HOMB_STAGE(5)
+      HOMB_STAGE(7)
+      HOMB_STAGE(11)
+      HOMB_STAGE(13)
+      HOMB_STAGE(9)
+      HOMB_STAGE(15)
+      default:
+        {
+          int qn = (R - 1) / 2, sn = (R - 1) / 2;
+          if (DIR > 0 && (band.prune & 1) && i == 0)   // pairs with a position <= half or >= M - top
+            qn = pairs_in_band(qn, nb, band);
+          if (DIR < 0 && (band.prune & 2) && i == plan.nrad - 1)
+            sn = pairs_in_band(sn, Ns, band);
+          stage_prime_sums<T, DIR>(src, G, ld, M, R, Ns, qn, dnb, dns, W);
+          __syncthreads();
+          stage_prime_out<T, DIR>(src, dst, G, ld, M, R, Ns, qn, sn, dnb, dns, W);
+        }
+        break;
+    }
+#undef HOMB_STAGE
+    __syncthreads();
+    cpx<T>* t = src; src = dst; dst = t;
+    Ns *= R;
+  }
+  return src;
+}
+
+template <typename T>
+__device__ cpx<T>* fft_pencils(cpx<T>* a, cpx<T>* b, int G, int ld, const FftPlan& plan, const cpx<T>* W, int dir,
+                               FftBand band = FftBand{0, 0, 0}) {
+  return dir > 0 ? fft_plan_run<T, 1>(a, b, G, ld, plan, W, band) : fft_plan_run<T, -1>(a, b, G, ld, plan, W, band);
+}
+
+// The batched kernel's form of fft_pencils, for plans of radices 3 to 13 alone. A batch has no
+// FP64 refinement, so its bounds at a loose tolerance carry the rounding of its FP32 CG: with
+// the order of operations of fft_pencils they moved by 1.2e-9, and by 6e-7 where a cell
+// stops at its FP32 floor (cells of one odd N, tolerance 1e-4). So this form keeps its
+// arithmetic operation by operation (stages in the plan's order, radices 7 to 13 as direct
+// sums, a direction known at run time only, which leaves no products to contract) and takes
+// only the multiplications for its divisions.
 template <typename T, int R>
-__device__ __forceinline__ void dftR(cpx<T>* v, const cpx<T>* W, int M, int dir) {
+__device__ __forceinline__ void dft_direct(cpx<T>* v, const cpx<T>* W, int M, int dir) {
   cpx<T> o[R];
   const int step = M / R;
 #pragma unroll
@@ -425,55 +818,29 @@ __device__ __forceinline__ void dftR(cpx<T>* v, const cpx<T>* W, int M, int dir)
 #pragma unroll
   for (int s = 0; s < R; ++s) v[s] = o[s];
 }
-
-// One Stockham stage for butterfly j of one pencil (src/dst of length M).
 template <typename T, int R>
-__device__ __forceinline__ void stage_bfly(const cpx<T>* __restrict__ src, cpx<T>* __restrict__ dst,
-                                           int j, int Ns, int M, const cpx<T>* W, int dir) {
+__device__ __forceinline__ void stage_small(const cpx<T>* __restrict__ src, cpx<T>* __restrict__ dst, int j, int Ns,
+                                            int M, DivConst dns, const cpx<T>* W, int dir) {
   const int nb = M / R;
-  const int k = j % Ns;
+  const int c = div_by(dns, j);
+  const int k = j - c * Ns;
   cpx<T> v[R];
 #pragma unroll
   for (int q = 0; q < R; ++q) v[q] = src[j + q * nb];
-  const int tstep = k * (M / (Ns * R));
+  const int tstep = k * (nb / Ns);
   if (k) {
 #pragma unroll
     for (int q = 1; q < R; ++q) v[q] = mulc<T>(v[q], W[q * tstep], dir > 0);
   }
   if (R == 3) dft3<T>(v, dir);
   else if (R == 5) dft5<T>(v, dir);
-  else dftR<T, R>(v, W, M, dir);
-  const int base = (j / Ns) * Ns * R + k;
+  else dft_direct<T, R>(v, W, M, dir);
+  const int base = c * Ns * R + k;
 #pragma unroll
   for (int q = 0; q < R; ++q) dst[base + q * Ns] = st_norm<T>(v[q]);
 }
-
-// Runtime radix (2 or a prime above 13) straight from shared memory: output s of butterfly j,
-// O(R) per output, so that a large prime radix spreads over R threads.
 template <typename T>
-__device__ void stage_out_generic(const cpx<T>* __restrict__ src, cpx<T>* __restrict__ dst,
-                                  int j, int s, int Ns, int M, int R, const cpx<T>* W, int dir) {
-  const int nb = M / R;
-  const int k = j % Ns;
-  const int tstep = k * (M / (Ns * R));
-  const int step = M / R;
-  const int base = (j / Ns) * Ns * R + k;
-  cpx<T> acc = src[j];
-  int ws = 0;   // (q * s) mod R, advanced incrementally
-  for (int q = 1; q < R; ++q) {
-    ws += s;
-    if (ws >= R) ws -= R;
-    const cpx<T> vq = mulc<T>(src[j + q * nb], W[q * tstep], dir > 0);
-    acc = add<T>(acc, mulc<T>(vq, W[ws * step], dir > 0));
-  }
-  dst[base + s * Ns] = st_norm<T>(acc);
-}
-
-// G pencils of length M at a + g*ld (ping-pong with b, same strides). The CTA runs
-// all stages; returns the buffer holding the result. Ends with __syncthreads().
-template <typename T>
-__device__ cpx<T>* fft_pencils(cpx<T>* a, cpx<T>* b, int G, int ld, const FftPlan& plan,
-                               const cpx<T>* W, int dir) {
+__device__ cpx<T>* fft_pencils_small(cpx<T>* a, cpx<T>* b, int G, int ld, const FftPlan& plan, const cpx<T>* W, int dir) {
   const int M = plan.M;
   int Ns = 1;
   cpx<T>* src = a;
@@ -481,30 +848,19 @@ __device__ cpx<T>* fft_pencils(cpx<T>* a, cpx<T>* b, int G, int ld, const FftPla
   for (int s = 0; s < plan.nrad; ++s) {
     const int R = plan.radix[s];
     const int nb = M / R;
-    if (R == 3 || R == 5 || R == 7 || R == 11 || R == 13) {
-      const int total = G * nb;
-      for (int t = threadIdx.x; t < total; t += blockDim.x) {
-        const int g = t / nb;
-        const int j = t - g * nb;
-        const cpx<T>* sp = src + (size_t)g * ld;
-        cpx<T>* dp = dst + (size_t)g * ld;
-        switch (R) {
-          case 3: stage_bfly<T, 3>(sp, dp, j, Ns, M, W, dir); break;
-          case 5: stage_bfly<T, 5>(sp, dp, j, Ns, M, W, dir); break;
-          case 7: stage_bfly<T, 7>(sp, dp, j, Ns, M, W, dir); break;
-          case 11: stage_bfly<T, 11>(sp, dp, j, Ns, M, W, dir); break;
-          default: stage_bfly<T, 13>(sp, dp, j, Ns, M, W, dir); break;
-        }
-      }
-    } else {
-      const int per = nb * R;
-      const int total = G * per;
-      for (int t = threadIdx.x; t < total; t += blockDim.x) {
-        const int g = t / per;
-        const int rem = t - g * per;
-        const int j = rem / R;
-        const int so = rem - j * R;
-        stage_out_generic<T>(src + (size_t)g * ld, dst + (size_t)g * ld, j, so, Ns, M, R, W, dir);
+    const bool have = plan.ndiv > 0;
+    const DivConst dnb = have ? plan.nb[s] : div_const((uint32_t)nb), dns = have ? plan.nsi[s] : div_const((uint32_t)Ns);
+    for (int t = threadIdx.x; t < G * nb; t += blockDim.x) {
+      const int g = div_by(dnb, t);
+      const int j = t - g * nb;
+      const cpx<T>* sp = src + (size_t)g * ld;
+      cpx<T>* dp = dst + (size_t)g * ld;
+      switch (R) {
+        case 3: stage_small<T, 3>(sp, dp, j, Ns, M, dns, W, dir); break;
+        case 5: stage_small<T, 5>(sp, dp, j, Ns, M, dns, W, dir); break;
+        case 7: stage_small<T, 7>(sp, dp, j, Ns, M, dns, W, dir); break;
+        case 11: stage_small<T, 11>(sp, dp, j, Ns, M, dns, W, dir); break;
+        default: stage_small<T, 13>(sp, dp, j, Ns, M, dns, W, dir); break;
       }
     }
     __syncthreads();

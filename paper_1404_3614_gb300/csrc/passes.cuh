@@ -35,9 +35,10 @@ __device__ __forceinline__ void stage_twiddles(cpx<T>* Ws, const void* W, int M)
 
 template <typename T, int MT>
 __device__ __forceinline__ cpx<T>* fft_any(cpx<T>* a, cpx<T>* b, int G, const FftPlan& plan,
-                                           const cpx<T>* W, int dir, int prune = 0) {
+                                           const cpx<T>* W, int dir, int prune = 0,
+                                           FftBand band = FftBand{0, 0, 0}) {
   if constexpr (MT > 0) return cfft<T, MT>(a, b, G, W, dir, prune);
-  else return fft_pencils<T>(a, b, G, plan.M, plan, W, dir);
+  else return fft_pencils<T>(a, b, G, plan.M, plan, W, dir, band);
 }
 
 // FP32 and float-float pencils of length 225 = 15 * 15 are transformed by warp-level
@@ -186,7 +187,8 @@ __global__ void __launch_bounds__(kPassThreads) k_pencil(PencilArgs a) {
     const bool zb = zero_band_free(M, a.Nlog);
     const int prune = (pad && prune3_ok(M, half + 1) ? 1 : 0) | (trunc_ && prune3_ok(M, half + 1) ? 2 : 0) |
                       (pad && zb ? 4 : 0) | (trunc_ && zb ? 8 : 0);
-    res = fft_any<T, MT>(A, B, XC, a.plan, Ws, a.dir, prune);
+    res = fft_any<T, MT>(A, B, XC, a.plan, Ws, a.dir, prune,
+                         FftBand{half, a.Nlog - 1 - half, (pad ? 1 : 0) | (trunc_ ? 2 : 0)});
   }
   cpx<T>* out = reinterpret_cast<cpx<T>*>(a.out) + (long long)s * a.out_slab;
   const bool trunc = a.dir < 0 && a.Pout != M;
@@ -256,7 +258,8 @@ __global__ void __launch_bounds__(kPassThreads) k_final(FinalArgs a) {
   } else {
     res = fft_any<T, MT>(A, B, C * XC, a.plan, Ws, -1,
                          (prune3_ok(M, (a.Nlog - 1) / 2 + 1) ? 2 : 0) |
-                             (a.Nlog < M && zero_band_free(M, a.Nlog) ? 8 : 0));
+                             (a.Nlog < M && zero_band_free(M, a.Nlog) ? 8 : 0),
+                         FftBand{(a.Nlog - 1) / 2, a.Nlog - 1 - (a.Nlog - 1) / 2, a.Nlog < M ? 2 : 0});
   }
   cpx<T>* out = reinterpret_cast<cpx<T>*>(a.out) + (long long)rhs * C * a.out_comp;
   const cpx<T>* pdir = (a.cg && a.aux) ? reinterpret_cast<const cpx<T>*>(a.aux) + (long long)rhs * C * a.out_comp
@@ -582,7 +585,8 @@ __global__ void __launch_bounds__(kPassThreads) k_xpass(XArgs a) {
   __syncthreads();
   cpx<T>* res = fft_any<T, MT>(A, B, npair, a.plan, Ws, +1,
                                a.mode != 2 ? ((prune3_ok(M, Nin) ? 1 : 0) | (zero_band_free(M, 2 * Nin - 1) ? 4 : 0))
-                                           : 0);
+                                           : 0,
+                               FftBand{Nin - 1, Nin - 1, a.mode != 2 && 2 * Nin - 1 < M ? 1 : 0});
   cpx<T>* oth = res == A ? B : A;
   const T* coef = reinterpret_cast<const T*>(a.coef);
   const long long cstride = (long long)a.planes * M;
@@ -611,7 +615,8 @@ __global__ void __launch_bounds__(kPassThreads) k_xpass(XArgs a) {
     }
     __syncthreads();
     cpx<T>* r2 = fft_any<T, MT>(res, oth, npair, a.plan, Ws, -1,
-                                (prune3_ok(M, a.Nout) ? 2 : 0) | (zero_band_free(M, 2 * a.Nout - 1) ? 8 : 0));
+                                (prune3_ok(M, a.Nout) ? 2 : 0) | (zero_band_free(M, 2 * a.Nout - 1) ? 8 : 0),
+                                FftBand{a.Nout - 1, a.Nout - 1, 2 * a.Nout - 1 < M ? 2 : 0});
     cpx<T>* out = reinterpret_cast<cpx<T>*>(a.out);
     const int Nout = a.Nout;
     for (int t = threadIdx.x; t < nrow * Nout; t += blockDim.x) {
