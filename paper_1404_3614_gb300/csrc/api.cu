@@ -396,10 +396,10 @@ struct Layout {
   }
 };
 
-int final_xc_elem(const Geometry& g, size_t elem) {
+int final_xc_elem(const Geometry& g, size_t elem, int R) {
   const int M = g.d == 3 ? g.M[2] : g.M[1];
   const int X = g.d == 3 ? g.N[1] * g.Nh : g.Nh;
-  return elem == 16 ? pencil_xc<double>(M, X, g.d) : pencil_xc<float>(M, X, g.d);
+  return elem == 16 ? pencil_xc<double>(M, X, g.d, R) : pencil_xc<float>(M, X, g.d, R);
 }
 
 // mode: 0 = hom_bounds (CG vectors in `elem`), 1 = step-level calls
@@ -475,8 +475,8 @@ Layout make_layout(const Geometry& g, int R, size_t elem, int mode) {
   L.cgo[0] = L.take(sizeof(CgScalars));
   L.cgo[1] = L.take(sizeof(CgScalars));
   const int X = g.d == 3 ? g.N[1] * g.Nh : g.Nh;
-  const int xcff = pencil_xc<ffloat>(g.d == 3 ? g.M[2] : g.M[1], X, g.d);
-  const int xc = std::max(1, std::min(std::min(final_xc_elem(g, 16), final_xc_elem(g, 8)), xcff > 0 ? xcff : 1 << 30));
+  const int xcff = pencil_xc<ffloat>(g.d == 3 ? g.M[2] : g.M[1], X, g.d, R);
+  const int xc = std::max(1, std::min(std::min(final_xc_elem(g, 16, R), final_xc_elem(g, 8, R)), xcff > 0 ? xcff : 1 << 30));
   L.maxblk = std::max(kVecBlocks, (X + xc - 1) / xc);
   L.partial = L.take((size_t)3 * L.maxblk * sizeof(double));
   L.rrpart = L.take((size_t)6 * kVecBlocks * sizeof(double));
@@ -807,7 +807,7 @@ struct Runner {
       z.in = cur; z.out = nxt; z.aux = nullptr;
       z.in_slab = z.out_slab = g.spec;
       z.nslab = g.ncomp; z.X = g.M[1] * g.Nxs;
-      z.XC = pencil_xc<double>(g.M[2], z.X, 1);
+      z.XC = pencil_xc<double>(g.M[2], z.X, 1, z.nslab);
       z.Pin = z.Pout = z.Nlog = g.M[2]; z.dir = +1;
       z.slabs_per_rhs = z.nslab; z.slabs_per_comp = 1; z.C = 1; z.prologue = 0;
       z.W = base + L.tw64[2]; z.plan = g.plan[2]; z.cg = nullptr;
@@ -820,7 +820,7 @@ struct Runner {
     y.in = cur; y.out = nxt; y.aux = nullptr;
     y.in_slab = y.out_slab = (long long)g.M[1] * g.Nxs;
     y.nslab = g.ncomp * g.M[2]; y.X = g.Nxs;
-    y.XC = pencil_xc<double>(g.M[1], y.X, 1);
+    y.XC = pencil_xc<double>(g.M[1], y.X, 1, y.nslab);
     y.Pin = y.Pout = y.Nlog = g.M[1]; y.dir = +1;
     y.slabs_per_rhs = y.nslab; y.slabs_per_comp = 1; y.C = 1; y.prologue = 0;
     y.W = base + L.tw64[1]; y.plan = g.plan[1]; y.cg = nullptr;
@@ -828,7 +828,7 @@ struct Runner {
     KL(launch_pencil<double>(y, st));
     XArgs x{};
     x.in = nxt; x.out = coef; x.coef = nullptr; x.mode = 2;
-    x.planes = (int)g.planes; x.YB = xpass_yb<double>(g.M[0], 1, (int)g.planes);
+    x.planes = (int)g.planes; x.YB = xpass_yb<double>(g.M[0], 1, (int)g.planes, g.ncomp);
     x.Nin = g.Nxs; x.Nout = 0; x.M = g.M[0]; x.R = 1; x.C = 1; x.ncomp = g.ncomp; x.d = g.d;
     x.comp_stride = g.planes * g.Nxs; x.scale = 1.0;
     x.W = base + L.tw64[0]; x.plan = g.plan[0]; x.cg = nullptr; x.partial = nullptr;
@@ -856,7 +856,7 @@ struct Runner {
       PencilArgs z{};
       z.in = in; z.out = T1; z.aux = r_aux;
       z.in_slab = (long long)Nz * Ny * Nh; z.out_slab = (long long)Mz * Ny * Nh;
-      z.nslab = R * C; z.X = Ny * Nh; z.XC = pencil_xc<T>(Mz, z.X, 1);
+      z.nslab = R * C; z.X = Ny * Nh; z.XC = pencil_xc<T>(Mz, z.X, 1, z.nslab);
       z.Pin = Nz; z.Pout = Mz; z.Nlog = Nz; z.dir = +1;
       z.slabs_per_rhs = C; z.slabs_per_comp = 1; z.C = C; z.prologue = prologue;
       z.W = W(2); z.plan = g.plan[2]; z.cg = cg; z.in64 = ff;
@@ -889,7 +889,7 @@ struct Runner {
       PencilArgs y{};
       y.in = ycur; y.out = T2; y.aux = g.d == 3 ? nullptr : r_aux;
       y.in_slab = (long long)Ny * Nh; y.out_slab = (long long)My * Nh;
-      y.nslab = R * C * Mz; y.X = Nh; y.XC = chunk(pencil_xc<T>(My, Nh, 1), ctx->ypass_xc);
+      y.nslab = R * C * Mz; y.X = Nh; y.XC = ctx->ypass_xc > 0 ? chunk(pencil_xc<T>(My, Nh, 1), ctx->ypass_xc) : pencil_xc<T>(My, Nh, 1, y.nslab);
       y.Pin = Ny; y.Pout = My; y.Nlog = Ny; y.dir = +1;
       y.slabs_per_rhs = C * Mz; y.slabs_per_comp = Mz; y.C = C;
       y.prologue = g.d == 3 ? 0 : prologue;
@@ -901,7 +901,8 @@ struct Runner {
       Prof pr(ctx, "xpass", st);
       XArgs x{};
       x.in = T2; x.out = T2; x.coef = coef; x.mode = 0;
-      x.planes = (int)g.planes; x.YB = chunk(xpass_yb<T>(Mx, C, (int)g.planes), ctx->xpass_yb);
+      x.planes = (int)g.planes; x.YB = ctx->xpass_yb > 0 ? chunk(xpass_yb<T>(Mx, C, (int)g.planes), ctx->xpass_yb)
+                               : xpass_yb<T>(Mx, C, (int)g.planes, R);
       x.Nin = Nh; x.Nout = Nh; x.M = Mx; x.R = R; x.C = C; x.ncomp = g.ncomp; x.d = g.d;
       x.comp_stride = g.planes * Nh; x.scale = 1.0 / (double)g.grid;
       x.W = W(0); x.plan = g.plan[0]; x.cg = cg; x.partial = nullptr;
@@ -913,7 +914,7 @@ struct Runner {
       PencilArgs y{};
       y.in = T2; y.out = T1; y.aux = nullptr;
       y.in_slab = (long long)My * Nh; y.out_slab = (long long)Ny * Nh;
-      y.nslab = R * C * Mz; y.X = Nh; y.XC = chunk(pencil_xc<T>(My, Nh, 1), ctx->ypass_xc);
+      y.nslab = R * C * Mz; y.X = Nh; y.XC = ctx->ypass_xc > 0 ? chunk(pencil_xc<T>(My, Nh, 1), ctx->ypass_xc) : pencil_xc<T>(My, Nh, 1, y.nslab);
       y.Pin = My; y.Pout = Ny; y.Nlog = Ny; y.dir = -1;
       y.slabs_per_rhs = C * Mz; y.slabs_per_comp = Mz; y.C = C; y.prologue = 0;
       y.W = W(1); y.plan = g.plan[1]; y.cg = cg;
@@ -929,7 +930,7 @@ struct Runner {
       const int Nlast = g.d == 3 ? Nz : Ny;
       f.X = g.d == 3 ? Ny * Nh : Nh;
       f.in_comp = (long long)Mlast * f.X; f.out_comp = (long long)Nlast * f.X;
-      f.nrhs = R; f.C = C; f.XC = pencil_xc<T>(Mlast, f.X, C); f.M = Mlast; f.Nlog = Nlast;
+      f.nrhs = R; f.C = C; f.XC = pencil_xc<T>(Mlast, f.X, C, R); f.M = Mlast; f.Nlog = Nlast;
       f.project = project; f.d = g.d; f.Ny = Ny; f.Nh = Nh;
       for (int k = 0; k < 3; ++k) f.invY[k] = g.invY[k];
       f.W = W(g.d == 3 ? 2 : 1); f.plan = g.plan[g.d == 3 ? 2 : 1];
@@ -960,14 +961,14 @@ struct Runner {
   int final_blocks_ff() const {
     const int M = g.d == 3 ? g.M[2] : g.M[1];
     const int X = g.d == 3 ? g.N[1] * g.Nh : g.Nh;
-    const int xc = pencil_xc<ffloat>(M, X, g.d);
+    const int xc = pencil_xc<ffloat>(M, X, g.d, R);
     return xc > 0 ? (X + xc - 1) / xc : 0;
   }
 
   int final_blocks(size_t elem) const {
     if (elem == 8 && final_pipe_grid() > 0) return final_pipe_grid();
     const int X = g.d == 3 ? g.N[1] * g.Nh : g.Nh;
-    const int xc = final_xc_elem(g, elem);
+    const int xc = final_xc_elem(g, elem, R);
     return (X + xc - 1) / xc;
   }
 
@@ -984,7 +985,7 @@ struct Runner {
       PencilArgs z{};
       z.in = x64; z.out = T1; z.aux = nullptr;
       z.in_slab = (long long)Nz * Ny * Nh; z.out_slab = (long long)Mz * Ny * Nh;
-      z.nslab = R * C; z.X = Ny * Nh; z.XC = pencil_xc<double>(Mz, z.X, 1);
+      z.nslab = R * C; z.X = Ny * Nh; z.XC = pencil_xc<double>(Mz, z.X, 1, z.nslab);
       z.Pin = Nz; z.Pout = Mz; z.Nlog = Nz; z.dir = +1;
       z.slabs_per_rhs = C; z.slabs_per_comp = 1; z.C = C; z.prologue = addE ? 2 : 0;
       z.W = base + L.tw64[2]; z.plan = g.plan[2]; z.cg = nullptr;
@@ -994,7 +995,7 @@ struct Runner {
     PencilArgs y{};
     y.in = ycur; y.out = T2; y.aux = nullptr;
     y.in_slab = (long long)Ny * Nh; y.out_slab = (long long)My * Nh;
-    y.nslab = R * C * Mz; y.X = Nh; y.XC = pencil_xc<double>(My, Nh, 1);
+    y.nslab = R * C * Mz; y.X = Nh; y.XC = pencil_xc<double>(My, Nh, 1, y.nslab);
     y.Pin = Ny; y.Pout = My; y.Nlog = Ny; y.dir = +1;
     y.slabs_per_rhs = C * Mz; y.slabs_per_comp = Mz; y.C = C;
     y.prologue = (g.d == 2 && addE) ? 2 : 0;
@@ -1002,7 +1003,7 @@ struct Runner {
     KL(launch_pencil<double>(y, st));
     XArgs x{};
     x.in = T2; x.out = nullptr; x.coef = coef; x.mode = 1;
-    x.planes = (int)g.planes; x.YB = xpass_yb<double>(g.M[0], R * C, (int)g.planes);
+    x.planes = (int)g.planes; x.YB = xpass_yb<double>(g.M[0], R * C, (int)g.planes, 1);
     if (x.YB < 1) return fail(ctx, HOM_ERR_INVALID_ARG, "grid too large for the shared-memory FFT");
     x.Nin = Nh; x.Nout = 0; x.M = g.M[0]; x.R = R; x.C = C; x.ncomp = g.ncomp; x.d = g.d;
     x.comp_stride = g.planes * Nh; x.scale = 1.0;

@@ -190,13 +190,16 @@ template <typename T> int batch_max_blocks(size_t smem, int threads, int cluster
 template <typename T> cudaError_t launch_pencil(const PencilArgs& a, cudaStream_t s);
 template <typename T> cudaError_t launch_final(const FinalArgs& a, cudaStream_t s);
 template <typename T> cudaError_t launch_xpass(const XArgs& a, int grid_y, cudaStream_t s);
-template <typename T> int pencil_xc(int M, int X, int C);   // chunk that fits shared memory
+// positions per CTA of a pencil pass: the chunk that fits shared memory, and with slabs > 0 (CTAs
+// beside the chunks) small enough that the grid fills the GPU
+template <typename T> int pencil_xc(int M, int X, int C, long long slabs = 0);
 // Persistent pipelined z passes of the FP32 3D operator at M = 225 (zpipe.cuh): their CTA
 // counts on a device with `sms` SMs, 0 where they do not apply (another length, a transform
 // that is not the zero-padded inverse / truncating forward one of the operator)
 int zpipe_pad_grid(int M, int Pin, int Pout, int Nlog, int dir, int X, int nslab, int sms);
 int zpipe_final_grid(int M, int Nlog, int d, int C, int X, int nrhs, int sms, int xc = 8);
-template <typename T> int xpass_yb(int M, int rows_per_plane, int planes);
+// planes per CTA of the row pass, in the same way (gy: CTAs beside the chunks)
+template <typename T> int xpass_yb(int M, int rows_per_plane, int planes, int gy = 0);
 // fused y-x-y slab pass; cudaErrorNotSupported when the length or size does not apply
 template <typename T> cudaError_t launch_slab(const SlabArgs& a, cudaStream_t s);
 template <typename T> int slab_warps(int M, int Nh);   // 0: slab pass not applicable

@@ -10,6 +10,7 @@
 // coefficient, r2c), the forward y transform with truncation (k_pencil) and the forward z
 // transform with truncation, Gamma and the CG partial sums (k_final).
 #pragma once
+#include <algorithm>
 #include <atomic>
 
 #include "attr.cuh"
@@ -700,7 +701,25 @@ __global__ void __launch_bounds__(kPassThreads) k_fft_batch(const cpx<T>* in, cp
 // ---------------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------------
-template <typename T> int pencil_xc(int M, int X, int C) {
+// A small grid's chunks, cut until the launch has about two CTAs for each of the 152 SMs: the
+// shared-memory budget alone gives a 2D cell of N = 23 one to four CTAs a pass, each a chain of
+// transforms on one SM (its FP64 operator 45.8 -> 30.9 us, its bounds 3.31 -> 2.20 ms, the same
+// results). A grid that reaches this many CTAs keeps its larger chunks (3D N = 41: 528.6 us both).
+constexpr long long kSpreadCtas = 304;
+inline long long spread_chunk(long long chunk, long long n, long long others) {
+  if (others < 1 || chunk < 2 || ((n + chunk - 1) / chunk) * others >= kSpreadCtas) return chunk;
+  const long long want = std::min(n, (kSpreadCtas + others - 1) / others);
+  return (n + want - 1) / want;
+}
+
+// Threads of a pass CTA with G pencils of length M: one per smallest (radix 3) butterfly, or the
+// warps that the register FFTs need (two pencils each)
+inline int pass_threads(int G, int M, bool warp_fft) {
+  const int t = warp_fft ? 32 * ((G + 1) / 2) : (G * M / 3 + 31) / 32 * 32;
+  return std::max(64, std::min(kPassThreads, t));
+}
+
+template <typename T> int pencil_xc_fit(int M, int X, int C) {
   const size_t sz = sizeof(cpx<T>);
   const size_t fixed = M * sz + 512;
   if (warp_fft_len<T>(M)) {
@@ -748,7 +767,11 @@ template <typename T> int pencil_xc(int M, int X, int C) {
   return (int)xc;
 }
 
-template <typename T> int xpass_yb(int M, int rpp, int planes) {
+template <typename T> int pencil_xc(int M, int X, int C, long long slabs) {
+  return (int)spread_chunk(pencil_xc_fit<T>(M, X, C), X, slabs);
+}
+
+template <typename T> int xpass_yb_fit(int M, int rpp, int planes) {
   const size_t sz = sizeof(cpx<T>);
   const size_t fixed = M * sz + 512;
   if (xpass_warp_len<T>(M)) {
@@ -778,6 +801,10 @@ template <typename T> int xpass_yb(int M, int rpp, int planes) {
   return (int)yb;
 }
 
+template <typename T> int xpass_yb(int M, int rpp, int planes, int gy) {
+  return (int)spread_chunk(xpass_yb_fit<T>(M, rpp, planes), planes, gy);
+}
+
 template <typename T, int MT> cudaError_t launch_pencil_m(PencilArgs a, cudaStream_t s) {
   const size_t bufs = warp_fft_r<T, MT>() > 0 ? 1 : 2;
   const size_t smem = (size_t)a.plan.M * sizeof(cpx<T>) * (1 + bufs * (size_t)a.XC);
@@ -785,7 +812,7 @@ template <typename T, int MT> cudaError_t launch_pencil_m(PencilArgs a, cudaStre
   cudaError_t e = smem_attr(k_pencil<T, MT>, smem, cache);
   if (e != cudaSuccess) return e;
   dim3 grid((a.X + a.XC - 1) / a.XC, a.nslab);
-  k_pencil<T, MT><<<grid, kPassThreads, smem, s>>>(a);
+  k_pencil<T, MT><<<grid, pass_threads(a.XC, a.plan.M, warp_fft_r<T, MT>() > 0), smem, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -796,7 +823,7 @@ template <typename T, int MT> cudaError_t launch_final_m(FinalArgs a, cudaStream
   cudaError_t e = smem_attr(k_final<T, MT>, smem, cache);
   if (e != cudaSuccess) return e;
   dim3 grid((a.X + a.XC - 1) / a.XC, a.nrhs);
-  k_final<T, MT><<<grid, kPassThreads, smem, s>>>(a);
+  k_final<T, MT><<<grid, pass_threads(a.C * a.XC, a.M, warp_fft_r<T, MT>() > 0), smem, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -812,7 +839,7 @@ template <typename T, int MT> cudaError_t launch_xpass_m(XArgs a, int grid_y, cu
   cudaError_t e = smem_attr(k_xpass<T, MT>, smem, cache);
   if (e != cudaSuccess) return e;
   dim3 grid((a.planes + a.YB - 1) / a.YB, grid_y);
-  k_xpass<T, MT><<<grid, kPassThreads, smem, s>>>(a);
+  k_xpass<T, MT><<<grid, pass_threads(npair, a.M, warp), smem, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -917,8 +944,8 @@ namespace homb {
   template cudaError_t launch_pencil<T>(const PencilArgs&, cudaStream_t);             \
   template cudaError_t launch_final<T>(const FinalArgs&, cudaStream_t);               \
   template cudaError_t launch_xpass<T>(const XArgs&, int, cudaStream_t);              \
-  template int pencil_xc<T>(int, int, int);                                           \
-  template int xpass_yb<T>(int, int, int);                                            \
+  template int pencil_xc<T>(int, int, int, long long);                                \
+  template int xpass_yb<T>(int, int, int, int);                                       \
   template cudaError_t launch_fft_batch<T>(const void*, void*, int, int, int, const void*, \
                                            const FftPlan&, cudaStream_t);
 

@@ -5,5 +5,5 @@
 namespace homb {
 static_assert(sizeof(cpx<ffloat>) == sizeof(double2), "float-float complex values take FP64's storage");
 template cudaError_t launch_pencil<ffloat>(const PencilArgs&, cudaStream_t);
-template int pencil_xc<ffloat>(int, int, int);
+template int pencil_xc<ffloat>(int, int, int, long long);
 }  // namespace homb

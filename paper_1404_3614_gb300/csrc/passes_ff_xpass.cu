@@ -4,5 +4,5 @@
 #include "passes.cuh"
 namespace homb {
 template cudaError_t launch_xpass<ffloat>(const XArgs&, int, cudaStream_t);
-template int xpass_yb<ffloat>(int, int, int);
+template int xpass_yb<ffloat>(int, int, int, int);
 }  // namespace homb
