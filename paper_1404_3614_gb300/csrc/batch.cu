@@ -14,6 +14,9 @@
 #include <cooperative_groups.h>
 #include <math.h>
 
+// the batch keeps its FP32 rounding (see fft_pencils_small): no packed complex operations, which
+// would also change which products are contracted
+#define HOMB_SCALAR_COMPLEX
 #include "attr.cuh"
 #include "kernels.cuh"
 #include "spectrum.cuh"
