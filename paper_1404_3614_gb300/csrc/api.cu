@@ -869,7 +869,7 @@ struct Runner {
     const void* fin = T2;
     bool use_slab = false;
     if constexpr (!ff)
-      use_slab = g.d == 3 && g.ncomp == 1 && g.M[0] == g.M[1] && ctx->slab_on && slab_warps<T>(g.M[0], Nh) > 0;
+      use_slab = g.d == 3 && g.ncomp == 1 && g.M[0] == g.M[1] && ctx->slab_on && slab_warps<T>(g.M[0], Ny, Nh) > 0;
     if (use_slab) {
       // fused inverse y, x row pass and forward y on each (rhs, comp, z) slab of T1
       if constexpr (!ff) {

@@ -202,7 +202,7 @@ int zpipe_final_grid(int M, int Nlog, int d, int C, int X, int nrhs, int sms, in
 template <typename T> int xpass_yb(int M, int rows_per_plane, int planes, int gy = 0);
 // fused y-x-y slab pass; cudaErrorNotSupported when the length or size does not apply
 template <typename T> cudaError_t launch_slab(const SlabArgs& a, cudaStream_t s);
-template <typename T> int slab_warps(int M, int Nh);   // 0: slab pass not applicable
+template <typename T> int slab_warps(int M, int Ny, int Nh);   // 0: slab pass not applicable
 
 cudaError_t launch_axis_tables(int nincl, int d, const int* M, int Mmax, const double* invY,
                                const DevIncl* incl, double2* phase, double* sinc, cudaStream_t s);

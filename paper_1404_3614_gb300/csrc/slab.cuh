@@ -13,30 +13,43 @@
 // the twiddles w_M^(l k2), exchanges through shared memory, and does the second register
 // DFT; lane l then holds X[l + R k1] (k1 < R). The output layout of the inverse x
 // transform is the input layout of the forward one, so the coefficient product happens
-// in registers between them.
+// in registers between them. In the slab kernel every lane group transforms two pencils at
+// once in packed FP32 arithmetic (fpair): two columns, or two pairs of rows.
 #pragma once
 #include <algorithm>
 
+#include "fpair.cuh"
 #include "kernels.cuh"
 
 namespace homb {
 
-constexpr int kSlabMaxThreads = 640;   // 20 warps: up to 102 registers a thread
+template <> struct cplx_t<fpair> { using type = fpair2; };
 
-// Byte offset of the scratch / staging region of a slab CTA: after the barrier (16 bytes),
-// the twiddles [M] and the slab [Nh][M], rounded up to 16 bytes (the bulk copy lands there).
-__host__ __device__ inline size_t slab_scratch_offset(int M, int Nh, size_t elem) {
-  return (16 + elem * ((size_t)M + (size_t)Nh * M) + 15) & ~(size_t)15;
+constexpr int kSlabMaxThreads = 480;   // 15 warps: up to 136 registers a thread
+
+// Layout of the slab in shared memory: columns kx = l + R m and l + R (m + 1), m even, side by side
+// (a column pair: one lane group's two pencils in the y passes, and two of a lane's values
+// in the x pass), each y position one 16-byte group (re, re', im, im'). Rows m < slab_rows hold
+// the Nh columns (those past Nh are zero); a pair's stride is odd and covers whole groups of four
+// rows, so that the x pass, eight lanes on eight pairs, has no bank conflicts.
+__host__ __device__ constexpr int slab_rows(int R, bool zb) {
+  return zb ? ((R * R + 3) / 4 + R - 1) / R : (R + 1) / 2;   // ZeroBand<R>::lo, or all of M = N
+}
+__host__ __device__ constexpr int slab_pairs(int R, bool zb) { return (slab_rows(R, zb) + 1) / 2 * R; }
+__host__ __device__ constexpr int slab_ld(int M) { return (M + 3) / 4 * 4 + 1; }
+
+// Byte offset of the scratch / staging region of a slab CTA: after the barrier (16 bytes), two
+// twiddle tables [M] and the column pairs (the bulk copy lands there).
+__host__ __device__ inline size_t slab_scratch_offset(int R, bool zb) {
+  return 16 + (size_t)((R * R + 1) / 2 * 2) * 16 + (size_t)slab_pairs(R, zb) * slab_ld(R * R) * 16;
 }
 
-// shared memory of one slab CTA with `warps` warps (R*R = M): the scratch region holds the
-// x pass's pencils or the staged input slab (Ny x Nh plus one element of alignment slack)
-inline size_t slab_smem_bytes(int M, int R, int Nh, int warps, size_t elem) {
-  const int Ny = (M + 1) / 2;
-  const size_t scratch = std::max((size_t)warps * (32 / R) * M, (size_t)Ny * Nh + 2);
-  return slab_scratch_offset(M, Nh, elem) + elem * scratch;
+// shared memory of one slab CTA with `warps` warps: the scratch region holds the x pass's double
+// pencils or the staged input slab (Ny x Nh plus one element of alignment slack)
+inline size_t slab_smem_bytes(int R, bool zb, int Ny, int Nh, int warps) {
+  return slab_scratch_offset(R, zb) +
+         std::max((size_t)warps * (32 / R) * R * R * 16, ((size_t)Ny * Nh + 2) * 8);
 }
-
 
 // First-stage DFT of a zero-padded inverse transform (inputs of the zero band not read) and
 // last-stage DFT of a truncating forward one (outputs of the band not computed)
@@ -82,24 +95,6 @@ __device__ __forceinline__ void pencil_fft_inplace(cpx<T>* p, int l, const cpx<T
     for (int k = 0; k < R; ++k) p[l + R * k] = st_norm<T>(v[k]);
   }
   __syncwarp();
-}
-
-// Second half of a register FFT whose first-stage results v (lane l, index k2) are
-// exchanged through the scratch pencil S of this lane group: on return v[k1] =
-// X[l + R k1]. Lanes with own = false (no lane group) touch no memory.
-template <typename T, int R>
-__device__ __forceinline__ void fft_finish(cpx<T>* v, cpx<T>* S, int l, const cpx<T>* Wt, int dir, bool own) {
-#pragma unroll
-  for (int k = 1; k < R; ++k) v[k] = mulc<T>(v[k], Wt[k * R + l], dir > 0);
-  __syncwarp();
-  if (own) {
-#pragma unroll
-    for (int k = 0; k < R; ++k) S[l + R * k] = st_norm<T>(v[k]);
-  }
-  __syncwarp();
-#pragma unroll
-  for (int n = 0; n < R; ++n) v[n] = own ? S[n + R * l] : mk<T>(T(0), T(0));
-  dft_reg<T, R>(v, dir);
 }
 
 constexpr long long kSlabSpinLimit = 1LL << 22;   // polls of the staged-copy barrier
@@ -201,42 +196,68 @@ __device__ __forceinline__ void pencil_fft_pad_inv(cpx<T>* p, int l, const cpx<T
   __syncwarp();
 }
 
-// fft_finish whose outputs of the zero band are not needed (a truncating forward transform)
-template <typename T, int R>
-__device__ __forceinline__ void fft_finish_zout(cpx<T>* v, cpx<T>* S, int l, const cpx<T>* Wt, bool own) {
+// Twiddles w_M^(l k) on the first-stage results (conj: inverse), both pencils alike
+template <int R>
+__device__ __forceinline__ void slab_twiddle(fpair2* v, const float2* Wt, int l, bool conj) {
 #pragma unroll
-  for (int k = 1; k < R; ++k) v[k] = mulc<T>(v[k], Wt[k * R + l], false);
+  for (int k = 1; k < R; ++k) {
+    const float2 w = Wt[k * R + l];
+    v[k] = mulc<fpair>(v[k], mk<fpair>(fpair(w.x), fpair(w.y)), conj);
+  }
+}
+// Transpose of a lane group's R x R values through its pencil of shared memory: v[k] of lane l
+// goes to v[l] of lane k (own = false: nothing written, the values read are not used)
+template <int R>
+__device__ __forceinline__ void slab_exchange(fpair2* v, fpair2* S, int l, bool own) {
   __syncwarp();
   if (own) {
 #pragma unroll
-    for (int k = 0; k < R; ++k) S[l + R * k] = st_norm<T>(v[k]);
+    for (int k = 0; k < R; ++k) S[l + R * k] = v[k];
   }
   __syncwarp();
 #pragma unroll
-  for (int n = 0; n < R; ++n) v[n] = own ? S[n + R * l] : mk<T>(T(0), T(0));
-  dft_reg_zout<T, R>(v, -1);
+  for (int n = 0; n < R; ++n) v[n] = S[n + R * l];
+}
+__device__ __forceinline__ fpair slab_shfl(fpair a, int src) {
+  return fpair(__shfl_sync(0xffffffffu, a.v.x, src), __shfl_sync(0xffffffffu, a.v.y, src));
 }
 
-template <typename T, int R, bool ZB>
+// 225^3, 9 components: 0.311 -> 0.275 ms a launch (the 3-field operator 428 -> 390 us) against one
+// pencil a lane group: 259 M -> 126 M warp instructions. It is bound by shared-memory
+// accesses now (72 % of the L1 data pipe; FP32 pipe 45 %, issue 39 %): a pencil passes through
+// shared memory once between its two register DFTs, and once between the y and x passes.
+template <int R, bool ZB>
 __global__ void __launch_bounds__(kSlabMaxThreads) k_slab(SlabArgs a) {
+  using F = fpair;
   constexpr int M = R * R;
-  constexpr int PW = 32 / R;   // pencils per warp
+  constexpr int LD = slab_ld(M);
+  constexpr int PW = 32 / R;   // lane groups per warp, two pencils each
+  constexpr int NM = slab_rows(R, ZB), NP = (NM + 1) / 2, NC = slab_pairs(R, ZB);
   extern __shared__ __align__(16) unsigned char smem[];
   uint64_t* mbar = reinterpret_cast<uint64_t*>(smem);
-  cpx<T>* Wt = reinterpret_cast<cpx<T>*>(smem + 16);
-  cpx<T>* P = Wt + M;                              // [Nh][M]: column kx, y contiguous
-  // x-pass scratch pencils [warps * PW][M], and between x passes the staged next input
-  cpx<T>* S = reinterpret_cast<cpx<T>*>(smem + slab_scratch_offset(M, a.Nh, sizeof(cpx<T>)));
+  float2* Wt = reinterpret_cast<float2*>(smem + 16);
+  float2* Ws = Wt + (M + 1) / 2 * 2;   // the same times 1 / (2 |M|)
+  fpair2* P = reinterpret_cast<fpair2*>(Ws + (M + 1) / 2 * 2);   // [NC][LD]
+  // x-pass scratch [warps * PW][M] double pencils, and between x passes the staged next input
+  float2* S = reinterpret_cast<float2*>(smem + slab_scratch_offset(R, ZB));
   const int Ny = a.Ny, Nh = a.Nh, half = (Ny - 1) / 2;
   const long long slab_elems = (long long)Ny * Nh;
   const long long nslabs = (long long)a.nrc * a.Mz;
-  const cpx<T>* in = reinterpret_cast<const cpx<T>*>(a.in);
-  cpx<T>* out = reinterpret_cast<cpx<T>*>(a.out);
+  const float2* in = reinterpret_cast<const float2*>(a.in);
+  float2* out = reinterpret_cast<float2*>(a.out);
   // twiddles w_M^(l k) stored at [k][l] so that the R lanes of a group read consecutive words
-  const cpx<T>* W = reinterpret_cast<const cpx<T>*>(a.W);
+  const float2* W = reinterpret_cast<const float2*>(a.W);
+  const float fs = 0.5f * (float)a.scale;   // 1 / |M| and the 1/2 of the split into rows
   for (int t = threadIdx.x; t < M; t += blockDim.x) {
     const int k = t / R;
-    Wt[t] = W[(t - k * R) * k];
+    const float2 w = W[(t - k * R) * k];
+    Wt[t] = w;
+    Ws[t] = make_float2(fs * w.x, fs * w.y);
+  }
+  // the padding rows M .. LD - 1 of every column pair: zero, and never written
+  for (int t = threadIdx.x; t < NC * (LD - M); t += blockDim.x) {
+    const int c = t / (LD - M);
+    P[c * LD + M + (t - c * (LD - M))] = mk<F>(F(0.f), F(0.f));
   }
   // slab q of the walk is (z, rc) = (q / nrc, q mod nrc) (z-major); in memory it is slab
   // rc * Mz + z of the [nrc][Mz][Ny][Nh] field
@@ -264,11 +285,11 @@ __global__ void __launch_bounds__(kSlabMaxThreads) k_slab(SlabArgs a) {
   }
   __syncthreads();
   // thread 0: start the staged copy of slab t; the plain end elements go to registers
-  cpx<T> edge0 = mk<T>(T(0), T(0)), edge1 = mk<T>(T(0), T(0));
+  float2 edge0 = make_float2(0.f, 0.f), edge1 = make_float2(0.f, 0.f);
   auto issue = [&](long long t) {
-    const cpx<T>* src = in + mem(t) * slab_elems;
-    const SlabStage st = slab_stage_plan<T>(src, slab_elems);
-    cpx<T>* stage = S + st.head;   // S is 16-byte aligned: element `head` lands aligned
+    const float2* src = in + mem(t) * slab_elems;
+    const SlabStage st = slab_stage_plan<float>(src, slab_elems);
+    float2* stage = S + st.head;   // S is 16-byte aligned: element `head` lands aligned
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mb), "r"(st.body) : "memory");
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
                      slab_smem_u32(stage + st.head)),
@@ -280,18 +301,25 @@ __global__ void __launch_bounds__(kSlabMaxThreads) k_slab(SlabArgs a) {
   if (threadIdx.x == 0 && s < nslabs) issue(s);
   uint32_t phase = 0;
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int sub = lane / R, l = lane - sub * R;
-  const bool act = sub < PW;
-  const int slots = (blockDim.x >> 5) * PW;
-  const int slot = warp * PW + sub;
-  constexpr int npairs = (M + 1) / 2;
-  const T scale = T(a.scale);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarp = blockDim.x >> 5;
+  // R = 15: one lane group to each half warp (the hardware serves a 64-bit access half by half:
+  // groups on lanes 0-14 and 15-29 cost a third wavefront); else R lanes after one another
+  const int sub = R == 15 ? lane >> 4 : lane / R;
+  const int l0 = R == 15 ? sub << 4 : sub * R;
+  const bool act = sub < PW && lane - l0 < R;
+  const int l = act ? lane - l0 : 0;
+  const int lc = l > 0 ? R - l : 0;                      // the column of this lane's negative frequencies
+  const int mirror = act && l > 0 ? l0 + lc : lane;      // and the lane that holds them
+  const int slots = nwarp * PW;
+  const int slot = act ? warp * PW + sub : 0;
+  constexpr int nquad = (M + 3) / 4;     // groups of four rows (the last one holds M mod 4 = 1)
+  static_assert(M % 4 == 1, "rows of the last group");
+  fpair2* Sw = reinterpret_cast<fpair2*>(S) + (size_t)slot * M;
 
   while (s < nslabs) {
     const int z = (int)(s / a.nrc);
-    const SlabStage st = slab_stage_plan<T>(in + mem(s) * slab_elems, slab_elems);
-    const cpx<T>* stage = S + st.head;
+    const SlabStage st = slab_stage_plan<float>(in + mem(s) * slab_elems, slab_elems);
+    const float2* stage = S + st.head;
     // ---- wait for the staged input (bounded), complete its plain end elements
     const bool ok = __syncthreads_and(slab_wait(mb, phase) ? 1 : 0) != 0;
     if (!ok) {
@@ -302,105 +330,157 @@ __global__ void __launch_bounds__(kSlabMaxThreads) k_slab(SlabArgs a) {
     }
     phase ^= 1u;
     if (threadIdx.x == 0) {
-      if (st.head) const_cast<cpx<T>*>(stage)[0] = edge0;
-      if (st.tail) const_cast<cpx<T>*>(stage)[slab_elems - 1] = edge1;
+      if (st.head) const_cast<float2*>(stage)[0] = edge0;
+      if (st.tail) const_cast<float2*>(stage)[slab_elems - 1] = edge1;
     }
     __syncthreads();
 
-    // ---- inverse y transforms of the Nh columns: input rows from the staged slab
-    // (row-major [Ny][Nh]), zero padded to M, results into column kx of P
-    for (int c0 = 0; c0 < Nh; c0 += slots) {
-      if (c0 + warp * PW >= Nh) break;   // no column for this warp in this or a later round
-      const int kx = c0 + slot;
-      const bool on = act && kx < Nh;
-      cpx<T>* p = P + (size_t)(on ? kx : 0) * M;
-      cpx<T> v[R];
+    // ---- inverse y transforms, a column pair to each lane group: input rows from the staged
+    // slab (row-major [Ny][Nh]), zero padded to M; columns past Nh are zero
+    for (int c0 = 0; c0 < NC; c0 += slots) {
+      if (c0 + warp * PW >= NC) break;   // no pair for this warp in this or a later round
+      const int c = c0 + slot;
+      const bool on = act && c < NC;
+      const int mp = c / R;              // columns l' + R 2 mp and l' + R (2 mp + 1), l' = c mod R
+      const int ka = c - mp * R + 2 * R * mp, kb = ka + R;
+      const bool ona = on && ka < Nh, onb = on && kb < Nh;
+      fpair2* p = P + (size_t)(on ? c : 0) * LD;
+      fpair2 v[R];
 #pragma unroll
       for (int n = 0; n < R; ++n) {
         if (ZB && ZeroBand<R>::in(n)) continue;   // padding rows only
         const int pos = l + R * n;
         const int y = pos <= half ? pos : (pos >= M - half ? pos - M + Ny : -1);
-        v[n] = (on && y >= 0) ? stage[(size_t)y * Nh + kx] : mk<T>(T(0), T(0));
+        float2 u = make_float2(0.f, 0.f), w = u;
+        if (y >= 0 && ona) u = stage[y * Nh + ka];
+        if (y >= 0 && onb) w = stage[y * Nh + kb];
+        v[n] = mk<F>(F(u.x, w.x), F(u.y, w.y));
       }
-      if constexpr (ZB) dft_reg_zin<T, R>(v, +1);
-      else dft_reg<T, R>(v, +1);
-#pragma unroll
-      for (int k = 1; k < R; ++k) v[k] = mulc<T>(v[k], Wt[k * R + l], true);   // inverse: conjugate twiddles
+      if constexpr (ZB) dft_reg_zin<F, R>(v, +1);
+      else dft_reg<F, R>(v, +1);
+      slab_twiddle<R>(v, Wt, l, true);   // inverse: conjugate twiddles
+      slab_exchange<R>(v, p, l, on);
+      dft_reg<F, R>(v, +1);
       __syncwarp();
       if (on) {
 #pragma unroll
         for (int k = 0; k < R; ++k) p[l + R * k] = v[k];
       }
-      __syncwarp();
-#pragma unroll
-      for (int n = 0; n < R; ++n) v[n] = on ? p[n + R * l] : mk<T>(T(0), T(0));
-      dft_reg<T, R>(v, +1);
-      __syncwarp();
-      if (on) {
-#pragma unroll
-        for (int k = 0; k < R; ++k) p[l + R * k] = v[k];
-      }
-      __syncwarp();
     }
     __syncthreads();
 
-    // ---- x row pass: rows ya = 2 pr and yb = 2 pr + 1 packed as Z = X_a + i X_b
-    cpx<T>* Sw = S + (size_t)(act ? slot : 0) * M;
-    const T* coefz = reinterpret_cast<const T*>(a.coef) + (size_t)z * M * M;
-    for (int p0 = 0; p0 < npairs; p0 += slots) {
-      if (p0 + warp * PW >= npairs) break;   // no row pair for this warp
-      const int pr = p0 + slot;
-      const bool on = act && pr < npairs;
-      const int ya = 2 * pr, yb = 2 * pr + 1;
-      const bool hb = on && yb < M;
-      // coefficient rows first: their global loads overlap the gather and the inverse FFT
-      T ca[R], cb[R];
+    // ---- x row pass: rows y0 .. y0 + 3 as two complex pencils Z = X_a + i X_b
+    const float* coefz = reinterpret_cast<const float*>(a.coef) + (size_t)z * M * M;
+    for (int q0 = 0; q0 < nquad; q0 += slots) {
+      if (q0 + warp * PW >= nquad) break;   // no rows for this warp
+      const bool on = act && q0 + slot < nquad;
+      const int y0 = on ? 4 * (q0 + slot) : 0;
+      const bool four = y0 + 3 < M;         // else one row
+      fpair2 v[R];
+      {
+        // columns l + R m (frequency k = l + R m, value m) and R - l + R m (frequency
+        // -k' = M - (R - l) - R m, value R - 1 - m; lane 0: its columns R m are the frequencies
+        // -R m, value R - m)
+        const fpair2* pf = P + (size_t)l * LD + y0;
+        const fpair2* pc = P + (size_t)lc * LD + y0;
+        fpair2 zc[2 * NP];
 #pragma unroll
-      for (int k = 0; k < R; ++k) {
-        ca[k] = on ? __ldg(coefz + (size_t)ya * M + l + R * k) : T(0);
-        cb[k] = hb ? __ldg(coefz + (size_t)yb * M + l + R * k) : T(0);
-      }
-      cpx<T> v[R];
+        for (int h = 0; h < NP; ++h) {
+          const fpair2 q[4] = {pf[h * R * LD], pf[h * R * LD + 1], pf[h * R * LD + 2], pf[h * R * LD + 3]};
 #pragma unroll
-      for (int n = 0; n < R; ++n) {
-        if (ZB && ZeroBand<R>::in(n)) continue;   // frequencies of the padding only
-        const int k = l + R * n;
-        cpx<T> A = mk<T>(T(0), T(0)), B = mk<T>(T(0), T(0));
-        if (on) {
-          if (k < Nh) {
-            A = P[k * M + ya];
-            if (hb) B = P[k * M + yb];
-            if (k == 0) { A.y = T(0); B.y = T(0); }
-          } else if (k > M - Nh) {
-            A = conj_<T>(P[(M - k) * M + ya]);
-            if (hb) B = conj_<T>(P[(M - k) * M + yb]);
+          for (int e = 0; e < 2; ++e) {
+            const int n = 2 * h + e;
+            if (n >= NM) continue;
+            float re[4], im[4];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+              re[r] = e ? q[r].x.v.y : q[r].x.v.x;
+              im[r] = e ? q[r].y.v.y : q[r].y.v.x;
+              if (n == 0 && l == 0) im[r] = 0.f;
+            }
+            v[n] = mk<F>(F(re[0] - im[1], re[2] - im[3]), F(im[0] + re[1], im[2] + re[3]));
+          }
+          const fpair2 c[4] = {pc[h * R * LD], pc[h * R * LD + 1], pc[h * R * LD + 2], pc[h * R * LD + 3]};
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+            float re[4], im[4];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+              re[r] = e ? c[r].x.v.y : c[r].x.v.x;
+              im[r] = e ? c[r].y.v.y : c[r].y.v.x;
+            }
+            zc[2 * h + e] = mk<F>(F(re[0] + im[1], re[2] + im[3]), F(re[1] - im[0], re[3] - im[2]));
           }
         }
-        v[n] = mk<T>(A.x - B.y, A.y + B.x);
-      }
-      if constexpr (ZB) dft_reg_zin<T, R>(v, +1);
-      else dft_reg<T, R>(v, +1);
-      fft_finish<T, R>(v, Sw, l, Wt, +1, act);
-      // v[k1] = z(x = l + R k1): real part row ya, imaginary part row yb
 #pragma unroll
-      for (int k = 0; k < R; ++k) v[k] = mk<T>(v[k].x * (ca[k] * scale), v[k].y * (cb[k] * scale));
+        for (int m = 0; m < NM; ++m) {
+          const fpair2 up = m + 1 < NM ? zc[m + 1] : mk<F>(F(0.f), F(0.f));
+          const fpair2 w = l == 0 ? up : zc[m];
+          if (R - 1 - m >= NM) v[R - 1 - m] = w;
+          else if (R - 1 - m == m && l + R * m >= Nh) v[m] = w;   // M = N: the middle value, either side of Nh
+        }
+      }
+      if constexpr (ZB) dft_reg_zin<F, R>(v, +1);
+      else dft_reg<F, R>(v, +1);
+      // the coefficient of the even rows (real parts): loaded before the second half of the
+      // transform, so that it overlaps the exchange
+      const float* cy = coefz + (size_t)y0 * M + l;
+      const float* cy2 = four ? cy + 2 * M : cy;
+      F ce[R];
+#pragma unroll
+      for (int k = 0; k < R; ++k) ce[k] = F(__ldg(cy + R * k), __ldg(cy2 + R * k));
+      slab_twiddle<R>(v, Wt, l, true);
+      slab_exchange<R>(v, Sw, l, act);
+      dft_reg<F, R>(v, +1);
+      // v[k1] = z(x = l + R k1): real parts rows y0, y0 + 2, imaginary parts rows y0 + 1, y0 + 3
+      // (a group of one row has zeros in the others)
+#pragma unroll
+      for (int k = 0; k < R; ++k) v[k].x = v[k].x * ce[k];
+      const float* cy1 = four ? cy + M : cy;
+      const float* cy3 = four ? cy + 3 * M : cy;
+#pragma unroll
+      for (int k = 0; k < R; ++k) ce[k] = F(__ldg(cy1 + R * k), __ldg(cy3 + R * k));
+#pragma unroll
+      for (int k = 0; k < R; ++k) v[k].y = v[k].y * ce[k];
       // forward transform: lane l holds x[l + R n2] with n2 = k1; the kept frequencies only
-      dft_reg<T, R>(v, -1);
-      if constexpr (ZB) fft_finish_zout<T, R>(v, Sw, l, Wt, act);
-      else fft_finish<T, R>(v, Sw, l, Wt, -1, act);
-      __syncwarp();
-      if (act) {
+      dft_reg<F, R>(v, -1);
+      slab_twiddle<R>(v, Ws, l, false);
+      v[0] = scl<F>(v[0], F(fs));
+      slab_exchange<R>(v, Sw, l, act);
+      if constexpr (ZB) dft_reg_zout<F, R>(v, -1);
+      else dft_reg<F, R>(v, -1);
+      // split Z into its rows: Z(M - k), k = l + R n, is value R - 1 - n of the lane R - l, and of
+      // lane 0 its own value R - n
+      fpair2* d = P + (size_t)l * LD + y0;
 #pragma unroll
-        for (int k = 0; k < R; ++k)
-          if (!(ZB && ZeroBand<R>::in(k))) Sw[l + R * k] = v[k];
-      }
-      __syncwarp();
-      if (on) {
-        for (int kx = l; kx < Nh; kx += R) {
-          const cpx<T> zk = Sw[kx];
-          const cpx<T> zm = Sw[kx == 0 ? 0 : M - kx];
-          P[kx * M + ya] = mk<T>(T(0.5) * (zk.x + zm.x), T(0.5) * (zk.y - zm.y));
-          if (hb) P[kx * M + yb] = mk<T>(T(0.5) * (zk.y + zm.y), T(-0.5) * (zk.x - zm.x));
+      for (int h = 0; h < NP; ++h) {
+        float re[4][2], im[4][2];   // [row][column of the pair]
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const int n = 2 * h + e;
+          if (n >= NM) {
+#pragma unroll
+            for (int r = 0; r < 4; ++r) re[r][e] = im[r][e] = 0.f;
+            continue;
+          }
+          fpair2 zm;
+          zm.x = slab_shfl(v[R - 1 - n].x, mirror);
+          zm.y = slab_shfl(v[R - 1 - n].y, mirror);
+          if (l == 0) zm = v[n == 0 ? 0 : R - n];
+          const fpair2 zk = v[n];
+          re[0][e] = zk.x.v.x + zm.x.v.x;
+          im[0][e] = zk.y.v.x - zm.y.v.x;
+          re[1][e] = zk.y.v.x + zm.y.v.x;
+          im[1][e] = zm.x.v.x - zk.x.v.x;
+          re[2][e] = zk.x.v.y + zm.x.v.y;
+          im[2][e] = zk.y.v.y - zm.y.v.y;
+          re[3][e] = zk.y.v.y + zm.y.v.y;
+          im[3][e] = zm.x.v.y - zk.x.v.y;
+        }
+        if (on) {
+#pragma unroll
+          for (int r = 0; r < 4; ++r)
+            if (r == 0 || four) d[h * R * LD + r] = mk<F>(F(re[r][0], re[r][1]), F(im[r][0], im[r][1]));
         }
       }
       __syncwarp();
@@ -413,43 +493,58 @@ __global__ void __launch_bounds__(kSlabMaxThreads) k_slab(SlabArgs a) {
     const long long sn = next_active(s);
     if (threadIdx.x == 0 && sn < nslabs) issue(sn);
 
-    // ---- forward y transforms (truncated; with ZB the zero band's rows are neither computed nor
-    // stored)
-    for (int c0 = 0; c0 < Nh; c0 += slots) {
-      if (c0 + warp * PW >= Nh) break;
-      const int kx = c0 + slot;
-      const bool on = act && kx < Nh;
-      if constexpr (ZB) pencil_fft_fwd_trunc<T, R>(P + (size_t)(on ? kx : 0) * M, l, Wt, on);
-      else pencil_fft_inplace<T, R>(P + (size_t)(on ? kx : 0) * M, l, Wt, -1, on);
+    // ---- forward y transforms in place (truncated; with ZB the zero band's rows are neither
+    // computed nor stored)
+    for (int c0 = 0; c0 < NC; c0 += slots) {
+      if (c0 + warp * PW >= NC) break;
+      const bool on = act && c0 + slot < NC;
+      fpair2* p = P + (size_t)(on ? c0 + slot : 0) * LD;
+      fpair2 v[R];
+#pragma unroll
+      for (int n = 0; n < R; ++n) v[n] = p[l + R * n];
+      dft_reg<F, R>(v, -1);
+      slab_twiddle<R>(v, Wt, l, false);
+      slab_exchange<R>(v, p, l, on);
+      if constexpr (ZB) dft_reg_zout<F, R>(v, -1);
+      else dft_reg<F, R>(v, -1);
+      __syncwarp();
+      if (on) {
+#pragma unroll
+        for (int k = 0; k < R; ++k)
+          if (!(ZB && ZeroBand<R>::in(k))) p[l + R * k] = v[k];
+      }
     }
     __syncthreads();
-    cpx<T>* o = out + mem(s) * slab_elems;
-    for (int t = threadIdx.x; t < Ny * Nh; t += blockDim.x) {
-      const int y = t / Nh;
-      const int kx = t - y * Nh;
-      const int pos = y <= half ? y : y - Ny + M;
-      o[t] = P[kx * M + pos];
+    float2* o = out + mem(s) * slab_elems;
+    for (int kx = lane; kx < Nh; kx += 32) {
+      const int m = kx / R;
+      const float* pk = reinterpret_cast<const float*>(P + (size_t)(m / 2 * R + kx - m * R) * LD) + (m & 1);
+#pragma unroll 4
+      for (int y = warp; y < Ny; y += nwarp) {
+        const int pos = y <= half ? y : y - Ny + M;
+        o[(size_t)y * Nh + kx] = make_float2(pk[4 * pos], pk[4 * pos + 2]);
+      }
     }
     __syncthreads();   // P is rewritten by the next slab's inverse y transforms
     s = sn;
   }
 }
 
-template <typename T, int R, bool ZB> cudaError_t launch_slab_rz(const SlabArgs& a, int warps, cudaStream_t s) {
-  const size_t smem = slab_smem_bytes(R * R, R, a.Nh, warps, sizeof(cpx<T>));
+template <int R, bool ZB> cudaError_t launch_slab_rz(const SlabArgs& a, int warps, cudaStream_t s) {
+  const size_t smem = slab_smem_bytes(R, ZB, a.Ny, a.Nh, warps);
   static std::atomic<int> cache[kAttrDevices] = {};
-  cudaError_t e = smem_attr(k_slab<T, R, ZB>, smem, cache);
+  cudaError_t e = smem_attr(k_slab<R, ZB>, smem, cache);
   if (e != cudaSuccess) return e;
   // persistent: as many CTAs as are resident at once, at most one per slab
   int dev = 0, sms = 0, per = 0;
   e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_slab<T, R, ZB>, warps * 32, smem);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_slab<R, ZB>, warps * 32, smem);
   if (e != cudaSuccess) return e;
   if (per < 1) return cudaErrorInvalidConfiguration;
   const long long nslabs = (long long)a.nrc * a.Mz;
   const int grid = (int)std::min<long long>(nslabs, (long long)sms * per);
-  k_slab<T, R, ZB><<<grid, warps * 32, smem, s>>>(a);
+  k_slab<R, ZB><<<grid, warps * 32, smem, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -464,34 +559,31 @@ inline bool slab_band_free(int M, int Ny, int Nh) {
   return f(Ny) && f(2 * Nh - 1);
 }
 
-template <typename T, int R> cudaError_t launch_slab_r(const SlabArgs& a, int warps, cudaStream_t s) {
-  return slab_band_free(a.M, a.Ny, a.Nh) ? launch_slab_rz<T, R, true>(a, warps, s)
-                                         : launch_slab_rz<T, R, false>(a, warps, s);
+template <int R> cudaError_t launch_slab_r(const SlabArgs& a, int warps, cudaStream_t s) {
+  return slab_band_free(a.M, a.Ny, a.Nh) ? launch_slab_rz<R, true>(a, warps, s) : launch_slab_rz<R, false>(a, warps, s);
 }
 
 // Warps per slab CTA, or 0 when the slab pass does not apply (length not R*R with R in
 // {3, 5, 9, 15}, or the slab does not fit in shared memory).
-template <typename T> int slab_warps(int M, int Nh) {
+template <typename T> int slab_warps(int M, int Ny, int Nh) {
   int R = 0;
   for (int r : {3, 5, 9, 15})
     if (r * r == M) R = r;
   // FP64 stays on the separate passes: it is bound by the FP64 pipe, and lane groups of R
   // leave 32 mod R lanes of every warp issuing FP64 work on zeros
   if (R == 0 || sizeof(T) == 8) return 0;
-  const size_t elem = sizeof(cpx<T>);
-  // eight warps when at least two CTAs fit on an SM; else one CTA per SM with the fewest
-  // warps that reach the fewest rounds of lane-group tasks (two column rounds, weight 1
-  // each, plus row-pair rounds, weight 2.5), measured best at 225^3 (20 warps: 0.44 ms,
-  // 16: 0.47, 24: 0.47)
-  if (2 * slab_smem_bytes(M, R, Nh, 8, elem) <= 220 * 1024) return 8;
-  const int PW = 32 / R, npairs = (M + 1) / 2;
+  // the warps with the least idle lane groups over the rounds (two rounds of column pairs, weight 1
+  // each, and of row groups, weight 2.2), more warps where that ties: 225: 15, 81: 7, 25: 2, 9: 1
+  const bool zb = slab_band_free(M, Ny, Nh);
+  const int PW = 32 / R, nc = slab_pairs(R, zb), nquad = (M + 3) / 4;
   int best = 0;
   double best_cost = 1e30;
-  for (int w = 8; w * 32 <= kSlabMaxThreads; w += 4) {
-    if (slab_smem_bytes(M, R, Nh, w, elem) > 220 * 1024) break;
+  for (int w = 1; w * 32 <= kSlabMaxThreads; ++w) {
+    if (slab_smem_bytes(R, zb, Ny, Nh, w) > 220 * 1024) break;
     const int slots = w * PW;
-    const double cost = 2.0 * ((Nh + slots - 1) / slots) + 2.5 * ((npairs + slots - 1) / slots);
-    if (cost < best_cost - 1e-9) {
+    const double cost = w * (2.0 * ((nc + slots - 1) / slots) + 2.2 * ((nquad + slots - 1) / slots)) *
+                        (w < 4 && M >= 81 ? 2.0 : 1.0);
+    if (cost <= best_cost + 1e-9) {
       best_cost = cost;
       best = w;
     }
@@ -503,17 +595,17 @@ template <typename T> cudaError_t launch_slab(const SlabArgs& a, cudaStream_t s)
   if constexpr (sizeof(T) != 4) {
     return cudaErrorNotSupported;
   } else {
-    int warps = slab_warps<T>(a.M, a.Nh);
+    int warps = slab_warps<T>(a.M, a.Ny, a.Nh);
     if (warps && a.warps > 0) {   // a caller's choice, where it fits
       const int r = a.M == 225 ? 15 : (a.M == 81 ? 9 : (a.M == 25 ? 5 : 3));
-      if (a.warps * 32 <= kSlabMaxThreads && slab_smem_bytes(a.M, r, a.Nh, a.warps, sizeof(cpx<T>)) <= 220 * 1024)
+      if (a.warps * 32 <= kSlabMaxThreads && slab_smem_bytes(r, slab_band_free(a.M, a.Ny, a.Nh), a.Ny, a.Nh, a.warps) <= 220 * 1024)
         warps = a.warps;
     }
     switch (warps ? a.M : 0) {
-      case 9: return launch_slab_r<T, 3>(a, warps, s);
-      case 25: return launch_slab_r<T, 5>(a, warps, s);
-      case 81: return launch_slab_r<T, 9>(a, warps, s);
-      case 225: return launch_slab_r<T, 15>(a, warps, s);
+      case 9: return launch_slab_r<3>(a, warps, s);
+      case 25: return launch_slab_r<5>(a, warps, s);
+      case 81: return launch_slab_r<9>(a, warps, s);
+      case 225: return launch_slab_r<15>(a, warps, s);
       default: return cudaErrorNotSupported;
     }
   }
