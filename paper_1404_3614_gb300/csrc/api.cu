@@ -235,7 +235,7 @@ void inv3(const double* A, int d, double* out) {  // leading dim 3
 
 double pdist(double a, double b, double Y) {
   double t = std::fabs(a - b);
-  t = std::fmod(t, Y);
+  if (!(t < Y)) t = std::fmod(t, Y);   // t < Y is its own remainder
   return std::min(t, Y - t);
 }
 
