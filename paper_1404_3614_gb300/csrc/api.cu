@@ -2113,25 +2113,31 @@ hom_status hom_bounds_batched(hom_ctx* ctx, int32_t n, const hom_problem* probs,
   };
   // CTAs of one launch: as many as fit at once (0 when the cluster shape cannot be placed),
   // at most one per scratch slot, a multiple of the cluster size
-  auto grid_for = [&](int cap, int threads, int cluster, size_t* smem) {
+  auto grid_for = [&](int cap, int threads, int cluster, size_t* smem, bool cluster_slots = false) {
     *smem = batch_smem_bytes(bp.M0max, bp.M1max, cap, elem);
     const int mx = f32 ? batch_max_blocks<float>(*smem, threads, cluster)
                        : batch_max_blocks<double>(*smem, threads, cluster);
+    if (cluster_slots) return std::min(bp.nslots_max, mx / cluster) * cluster;
     const int g_ = std::min(bp.nslots_max, mx);
     return (g_ / cluster) * cluster;
   };
+  int run_stride = 0;
   int launched[6] = {0, 0, 0, 0, 0, 0};   // threads, cap, schedule, cluster, coopM, CTAs
   auto enqueue = [&](int cap, int threads, int cluster, int coopM, int max_iter) -> hom_status {
     size_t smem = 0;
-    int grid = grid_for(cap, threads, cluster, &smem);
+    bool cluster_slots = cluster > 1 && ncoop_for(cluster, coopM) == nt;
+    int grid = grid_for(cap, threads, cluster, &smem, cluster_slots);
     if (grid < cluster) {   // the cluster shape does not fit: single CTAs
+      cluster_slots = false;
       cluster = 1;
       grid = grid_for(cap, threads, 1, &smem);
     }
     if (grid < 1) return fail(ctx, HOM_ERR_INVALID_ARG, "batched kernel does not fit on the device");
     CK(h2d_copy(ctx, base + bp.o_tasks, ctx->pin_in, bp.in_bytes, st));
     CK(cudaMemsetAsync(base + bp.o_counter, 0, 2 * sizeof(int), st));
-    const BArgs a = args_for(cap, max_iter, ncoop_for(cluster, coopM));
+    BArgs a = args_for(cap, max_iter, ncoop_for(cluster, coopM));
+    a.cluster_slots = cluster_slots ? 1 : 0;
+    a.run_stride = run_stride;
     launched[0] = threads;
     launched[1] = cap;
     launched[3] = cluster;
@@ -2217,6 +2223,27 @@ hom_status hom_bounds_batched(hom_ctx* ctx, int32_t n, const hom_problem* probs,
     cudaEventDestroy(e1);
     ctx->tuned_cap.push_back({tkey, cap, threads, sched, cluster, coopM});
   }
+  if (!tuned && !opts->autotune && ctx->batch_threads == 0 && ctx->batch_cluster == 0) {
+    // Neither tuned nor chosen by the caller: every task on a cluster of 8 CTAs, so that no long
+    // task is left alone on one SM while the others idle. CTAs of 512 threads (15 clusters at
+    // once) where the longest task is a large part of a cluster's share of the batch, else 256
+    // (36 clusters). Against one 256-thread CTA a task: 64 cells of mixed N 235 -> 32 ms (512;
+    // 43 with 256), 24 of them 182 -> 22, 200 of them 262 -> 64 (256; 75 with 512), 63 cells of
+    // N = 89 164 -> 43 (256; 45), 16 of N = 113 28.7 -> 5.5 (512; 6.4). Cells up to N = 32 have
+    // too little work for 8 CTAs: clusters of 4 (64 cells of N = 23: 7.5 -> 6.7 ms, 7.5 with 8).
+    double work = 0.0, longest = 0.0;
+    for (const BTask& t : bp.tasks) {
+      const double w = (double)t.M0 * t.M1;
+      work += w;
+      longest = std::max(longest, w);
+    }
+    cluster = bp.Mmax <= 64 ? 4 : 8;
+    coopM = 0;
+    size_t sm_ = 0;
+    const int clusters = grid_for(cap, 256, cluster, &sm_, true) / cluster;
+    threads = cluster == 8 && work < 2.0 * clusters * longest ? 512 : 256;
+    run_stride = 256;
+  }
   set_sched(sched);
   if (ctx->batch_threads) threads = ctx->batch_threads;
   if (ctx->batch_cluster) {
@@ -2227,11 +2254,12 @@ hom_status hom_bounds_batched(hom_ctx* ctx, int32_t n, const hom_problem* probs,
   const int max_iter = opts->max_iter > 0 ? opts->max_iter : ((opts->max_iter == 0 && io && io->d_x0) ? 0 : 10000);
   if (opts->graph && st != nullptr) {
     size_t smem = 0;
-    const int grid = grid_for(cap, threads, cluster, &smem);
+    const int ncoop = ncoop_for(cluster, coopM);
+    const int grid = grid_for(cap, threads, cluster, &smem, cluster > 1 && ncoop == nt);
     const std::vector<long long> key = {(long long)threads, (long long)cluster, (long long)coopM,
                                         (long long)(uintptr_t)d_ws, (long long)(uintptr_t)(io ? io->d_x0 : nullptr),
                                         (long long)(uintptr_t)(io ? io->d_fields : nullptr),
-                                        (long long)bp.total, nt, grid, (long long)smem, cap,
+                                        (long long)bp.total, nt, ncoop, run_stride, grid, (long long)smem, cap,
                                         (long long)f32, max_iter, (long long)(tol * 1e18), (long long)ctx->pin_in_bytes,
                                         (long long)ctx->pin_out_bytes, bp.M0max, bp.M1max, bp.slot_bytes,
                                         (long long)ctx->batch_wpass};

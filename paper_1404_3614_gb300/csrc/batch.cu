@@ -429,7 +429,7 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 2 : 1) k_batch(BArgs a) {
       task = s_task;
       if (task >= a.ntasks) break;
     }
-    unsigned char* slot = a.slots + (long long)(blockIdx.x - tm.rank) * a.slot_bytes;
+    unsigned char* slot = a.slots + (long long)(a.cluster_slots ? blockIdx.x / csize : blockIdx.x - tm.rank) * a.slot_bytes;
     {
       // the task descriptor lives in shared memory (keeps the FFT plans out of registers)
       const int* src = reinterpret_cast<const int*>(a.tasks + task);
@@ -761,29 +761,42 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 2 : 1) k_batch(BArgs a) {
         const T al_ = T(s_alpha[r]);
         const long long o = (long long)r * n2f;
         double acc_r = 0.0;
-        float run = 0.f;   // FP32: runs of up to 8 terms, summed in FP64
-        int cnt = 0;
-        for (int i = tid0; i < n2f; i += nth) {
+        auto update = [&](int i) {
           const cpx<T> pv = vp[o + i], qv = vq[o + i];
           cpx<T> xv = vx[o + i], rv = vr[o + i];
           xv = mk<T>(fma(al_, pv.x, xv.x), fma(al_, pv.y, xv.y));
           rv = mk<T>(fma(-al_, qv.x, rv.x), fma(-al_, qv.y, rv.y));
           vx[o + i] = xv;
           vr[o + i] = rv;
-          const bool k0 = i - (int)fdNh.div(i) * Nh == 0;
-          if constexpr (sizeof(T) == 4) {
-            const float sq = fmaf(rv.x, rv.x, rv.y * rv.y);
-            run = fmaf(k0 ? 1.f : 2.f, sq, run);
-            if (++cnt == 8) {
-              acc_r += (double)run;
-              run = 0.f;
-              cnt = 0;
+          return rv;
+        };
+        if constexpr (sizeof(T) == 4) {
+          // runs of 8 terms in FP32, summed in FP64; the terms of a run lie run_stride entries
+          // apart (256 where the library chose the launch, so that every choice rounds alike; the
+          // team's threads else)
+          const int rs = a.run_stride > 0 ? a.run_stride : nth;
+          const int c0 = tid0 / rs;
+          for (int e = c0 * 8 * rs + (tid0 - c0 * rs); e < n2f; e += nth * 8) {
+            float run = 0.f;
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+              const int i = e + rs * u;
+              if (i >= n2f) break;
+              const cpx<T> rv = update(i);
+              const bool k0 = i - (int)fdNh.div(i) * Nh == 0;
+              const float sq = fmaf(rv.x, rv.x, rv.y * rv.y);
+              run = fmaf(k0 ? 1.f : 2.f, sq, run);
             }
-          } else {
+            acc_r += (double)run;
+          }
+        } else {
+          for (int i = tid0; i < n2f; i += nth) {
+            const cpx<T> rv = update(i);
+            const bool k0 = i - (int)fdNh.div(i) * Nh == 0;
             acc_r += (k0 ? 1.0 : 2.0) * ((double)rv.x * rv.x + (double)rv.y * rv.y);
           }
         }
-        rr[r] = acc_r + (double)run;
+        rr[r] = acc_r;
       }
       for (int r = 0; r < 2; ++r) {
         const double s = team_sum(tm, rr[r], s_red, s_xch, parity);

@@ -153,6 +153,8 @@ struct BArgs {
   int M0max, M1max;
   const void* x0;          // optional starting fields [prob][side][rhs][comp][N1][Nh] (working precision)
   void* fields;            // optional final CG fields, same layout
+  int run_stride;          // FP32 |r|^2: entries between the terms of a run (0: the team's threads)
+  int cluster_slots;       // every task is cooperative: one scratch slot per cluster
   int wpass;               // FP32: warp-owned pencil passes for 2N-1 in {45, 125, 225, 405}
 };
 
