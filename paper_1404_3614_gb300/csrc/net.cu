@@ -15,6 +15,7 @@
 #include <cuda_bf16.h>
 #include <math.h>
 
+#include <atomic>
 #include <cmath>
 #include <vector>
 
@@ -39,11 +40,13 @@ namespace homb {
 constexpr int TBM = 128, TBN = 64, TBK = 64;
 constexpr int kTmemCols = 64;                       // power of two >= 32
 constexpr int kTileABytes = TBM * TBK * 2, kTileBBytes = TBN * TBK * 2;
-// 26 KB of dynamic shared memory: at most 8 CTAs per SM (228 KB), 8 x 64 = 512 TMEM columns,
+// 27 KB of dynamic shared memory: at most 8 CTAs per SM (228 KB), 8 x 64 = 512 TMEM columns,
 // so an allocation never waits on a CTA that is not running
-constexpr int kGemmSmem = 26 * 1024;
-static_assert(kTileABytes + kTileBBytes + 16 <= kGemmSmem, "GEMM tiles exceed the shared-memory request");
-static_assert(TBM * 36 * 4 <= kTileABytes + kTileBBytes, "the result staging must fit in the operand tiles");
+constexpr int kGemmSmem = 27 * 1024;
+// layout: B tile, A tile (whose space, and a little more, stages the result), barrier
+constexpr int kStageOff = kTileBBytes, kBarOff = kTileBBytes + TBM * 36 * 4;
+static_assert(kBarOff + 16 <= kGemmSmem, "GEMM tiles exceed the shared-memory request");
+static_assert(kTileABytes <= TBM * 36 * 4, "the operand tile lies in the result staging");
 static_assert(TBN % 32 == 0, "the staged epilogue works in 32-column halves");
 constexpr long long kMbarSpinLimit = 1LL << 22;
 
@@ -97,18 +100,24 @@ __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t phase, long lo
   return false;
 }
 
-__global__ void __launch_bounds__(128) k_gemm(GemmArgs g, int ksplit, float* partial) {
+__device__ __forceinline__ float gelu(float x) { return 0.5f * x * (1.f + erff(x * 0.70710678118654752f)); }
+
+// PIPE: several chunks of K follow one another (a split of a long K): the next chunk's loads run
+// under this one's MMA, in registers (146 a thread). Else (K <= 64) a CTA walks row tiles with the
+// B tile staged once, eight CTAs an SM.
+template <bool PIPE>
+__global__ void __launch_bounds__(128, PIPE ? 3 : 8) k_gemm(GemmArgs g, int ksplit, float* partial) {
   extern __shared__ __align__(1024) unsigned char smem[];
-  unsigned char* sA = smem;                                 // [TBK/8][TBM/8][8][16 B]
-  unsigned char* sB = smem + kTileABytes;                   // [TBK/8][TBN/8][8][16 B]
-  uint64_t* mbar = reinterpret_cast<uint64_t*>(smem + kTileABytes + kTileBBytes);
+  unsigned char* sB = smem;                                 // [TBK/8][TBN/8][8][16 B]
+  unsigned char* sA = smem + kStageOff;                     // [TBK/8][TBM/8][8][16 B]
+  uint64_t* mbar = reinterpret_cast<uint64_t*>(smem + kBarOff);
   uint32_t* tslot = reinterpret_cast<uint32_t*>(mbar + 1);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int bz = blockIdx.z / ksplit;
   const int ks = blockIdx.z - bz * ksplit;
   const float* A = g.A + (long long)bz * g.sA;
   const float* B = g.B + (long long)bz * g.sB;
-  const int m0 = blockIdx.y * TBM, n0 = blockIdx.x * TBN;
+  const int n0 = blockIdx.x * TBN, mtiles = (g.M + TBM - 1) / TBM;
   const int kchunk = ((g.K + ksplit - 1) / ksplit + TBK - 1) / TBK * TBK;
   const int kbeg = ks * kchunk;
   const int kend = min(g.K, kbeg + kchunk);
@@ -130,47 +139,97 @@ __global__ void __launch_bounds__(128) k_gemm(GemmArgs g, int ksplit, float* par
   constexpr uint32_t idesc = mma_idesc(TBM, TBN);
   uint32_t phase = 0;
   bool ok = true;
-  for (int k0 = kbeg; k0 < kend && ok; k0 += TBK) {
-    // A tile: 8-element K runs of one row per store (16 bytes = one core-matrix row)
-    for (int c = tid; c < TBM * (TBK / 8); c += 128) {
-      int r, kc;
-      if (!g.ta) { r = c >> 3; kc = c & 7; }
-      else { r = c & (TBM - 1); kc = c / TBM; }
-      const int gm = m0 + r;
-      float v[8];
-      const int gk0 = k0 + kc * 8;
-      if (g.vecA && gm < g.M && gk0 + 8 <= kend) {   // two 16-byte loads along K
-        const float4* p = reinterpret_cast<const float4*>(A + (long long)gm * g.lda + gk0);
-        const float4 lo = __ldg(p), hi = __ldg(p + 1);
-        v[0] = lo.x; v[1] = lo.y; v[2] = lo.z; v[3] = lo.w; v[4] = hi.x; v[5] = hi.y; v[6] = hi.z; v[7] = hi.w;
-      } else {
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const int gk = gk0 + j;
-          v[j] = 0.f;
-          if (gm < g.M && gk < kend) v[j] = g.ta ? A[(long long)gk * g.lda + gm] : A[(long long)gm * g.lda + gk];
-        }
-      }
-      const uint4 q = make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]),
-                                 pack_bf16(v[6], v[7]));
-      *reinterpret_cast<uint4*>(sA + ((kc * (TBM / 8) + (r >> 3)) * 8 + (r & 7)) * 16) = q;
-    }
-    // B tile, stored N x K (K-major)
-    for (int c = tid; c < TBN * (TBK / 8); c += 128) {
-      int n, kc;
-      if (g.tb) { n = c >> 3; kc = c & 7; }
-      else { n = c & (TBN - 1); kc = c / TBN; }
-      const int gn = n0 + n;
-      float v[8];
+  // operand rows and columns that exist (the tile's others keep what is there: they reach no
+  // result), in tasks of one 8-element K run (16 bytes of BF16, one core-matrix row)
+  const int cols = min(TBN, g.N - n0), cols8 = (cols + 7) & ~7;
+  auto loadA = [&](float* v, int m0, int r, int kc, int k0) {
+    const int gm = m0 + r, gk0 = k0 + kc * 8;
+    if (g.vecA && gm < g.M && gk0 + 8 <= kend) {   // two 16-byte loads along K
+      const float4* p = reinterpret_cast<const float4*>(A + (long long)gm * g.lda + gk0);
+      const float4 lo = __ldg(p), hi = __ldg(p + 1);
+      v[0] = lo.x; v[1] = lo.y; v[2] = lo.z; v[3] = lo.w; v[4] = hi.x; v[5] = hi.y; v[6] = hi.z; v[7] = hi.w;
+    } else {
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
-        const int gk = k0 + kc * 8 + j;
+        const int gk = gk0 + j;
         v[j] = 0.f;
-        if (gn < g.N && gk < kend) v[j] = g.tb ? B[(long long)gn * g.ldb + gk] : B[(long long)gk * g.ldb + gn];
+        if (gm < g.M && gk < kend) v[j] = g.ta ? A[(long long)gk * g.lda + gm] : A[(long long)gm * g.lda + gk];
       }
-      const uint4 q = make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]),
-                                 pack_bf16(v[6], v[7]));
-      *reinterpret_cast<uint4*>(sB + ((kc * (TBN / 8) + (n >> 3)) * 8 + (n & 7)) * 16) = q;
+    }
+  };
+  auto loadB = [&](float* v, int n, int kc, int k0) {
+    const int gn = n0 + n;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const int gk = k0 + kc * 8 + j;
+      v[j] = 0.f;
+      if (gn < g.N && gk < kend) v[j] = g.tb ? B[(long long)gn * g.ldb + gk] : B[(long long)gk * g.ldb + gn];
+    }
+  };
+  auto pack = [](const float* v) {
+    return make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
+  };
+  constexpr int NA = TBM * (TBK / 8) / 128, NB = TBN * (TBK / 8) / 128;
+  float va[PIPE ? NA : 1][8], vb[PIPE ? NB : 1][8];
+  // task c of a tile of `lines` rows or columns: its line and its K group, of kcn
+  auto task = [](int c, bool along_k, int lines, int kcn, int& line, int& kc) {
+    if (along_k) { line = c / kcn; kc = c - line * kcn; }
+    else { kc = c / lines; line = c - kc * lines; }
+  };
+  bool haveB = false;
+  for (int mt = blockIdx.y; mt < mtiles && ok; mt += gridDim.y) {
+  const int m0 = mt * TBM;
+  const int rows8 = (min(TBM, g.M - m0) + 7) & ~7;
+  if (PIPE && kbeg < kend) {
+#pragma unroll
+    for (int t = 0; t < NA; ++t)
+      if (tid + t * 128 < rows8 * (TBK / 8)) {
+        int r, kc;
+        task(tid + t * 128, !g.ta, rows8, TBK / 8, r, kc);
+        loadA(va[PIPE ? t : 0], m0, r, kc, kbeg);
+      }
+#pragma unroll
+    for (int t = 0; t < NB; ++t)
+      if (tid + t * 128 < cols8 * (TBK / 8)) {
+        int n, kc;
+        task(tid + t * 128, g.tb, cols8, TBK / 8, n, kc);
+        loadB(vb[PIPE ? t : 0], n, kc, kbeg);
+      }
+  }
+  for (int k0 = kbeg; k0 < kend && ok; k0 += TBK) {
+    // 8-element K groups up to the MMA's multiple of 16
+    const int kcn = PIPE ? TBK / 8 : (min(TBK, kend - k0) + 15) / 16 * 2;
+    // A tile, and B stored N x K (K-major)
+    if constexpr (PIPE) {
+#pragma unroll
+      for (int t = 0; t < NA; ++t)
+        if (tid + t * 128 < rows8 * (TBK / 8)) {
+          int r, kc;
+          task(tid + t * 128, !g.ta, rows8, TBK / 8, r, kc);
+          *reinterpret_cast<uint4*>(sA + ((kc * (TBM / 8) + (r >> 3)) * 8 + (r & 7)) * 16) = pack(va[t]);
+        }
+#pragma unroll
+      for (int t = 0; t < NB; ++t)
+        if (tid + t * 128 < cols8 * (TBK / 8)) {
+          int n, kc;
+          task(tid + t * 128, g.tb, cols8, TBK / 8, n, kc);
+          *reinterpret_cast<uint4*>(sB + ((kc * (TBN / 8) + (n >> 3)) * 8 + (n & 7)) * 16) = pack(vb[t]);
+        }
+    } else {
+      for (int c = tid; c < rows8 * kcn; c += 128) {
+        int r, kc;
+        task(c, !g.ta, rows8, kcn, r, kc);
+        loadA(va[0], m0, r, kc, k0);
+        *reinterpret_cast<uint4*>(sA + ((kc * (TBM / 8) + (r >> 3)) * 8 + (r & 7)) * 16) = pack(va[0]);
+      }
+      if (!haveB)
+        for (int c = tid; c < cols8 * kcn; c += 128) {
+          int n, kc;
+          task(c, g.tb, cols8, kcn, n, kc);
+          loadB(vb[0], n, kc, k0);
+          *reinterpret_cast<uint4*>(sB + ((kc * (TBN / 8) + (n >> 3)) * 8 + (n & 7)) * 16) = pack(vb[0]);
+        }
+      haveB = true;
     }
     // make the generic-proxy stores visible to the tensor core (async proxy)
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -179,6 +238,7 @@ __global__ void __launch_bounds__(128) k_gemm(GemmArgs g, int ksplit, float* par
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
       for (int s = 0; s < TBK / 16; ++s) {
+        if (2 * s >= kcn) break;
         const uint64_t ad = smem_desc(smem_u32(sA) + s * 2 * (TBM / 8) * 128, (TBM / 8) * 128, 128);
         const uint64_t bd = smem_desc(smem_u32(sB) + s * 2 * (TBN / 8) * 128, (TBN / 8) * 128, 128);
         const uint32_t acc = (k0 > kbeg || s > 0) ? 1u : 0u;
@@ -190,6 +250,22 @@ __global__ void __launch_bounds__(128) k_gemm(GemmArgs g, int ksplit, float* par
       }
       asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar_a)
                    : "memory");
+    }
+    if (PIPE && k0 + TBK < kend) {
+#pragma unroll
+      for (int t = 0; t < NA; ++t)
+        if (tid + t * 128 < rows8 * (TBK / 8)) {
+          int r, kc;
+          task(tid + t * 128, !g.ta, rows8, TBK / 8, r, kc);
+          loadA(va[PIPE ? t : 0], m0, r, kc, k0 + TBK);
+        }
+#pragma unroll
+      for (int t = 0; t < NB; ++t)
+        if (tid + t * 128 < cols8 * (TBK / 8)) {
+          int n, kc;
+          task(tid + t * 128, g.tb, cols8, TBK / 8, n, kc);
+          loadB(vb[PIPE ? t : 0], n, kc, k0 + TBK);
+        }
     }
     ok = __syncthreads_and(mbar_wait(mbar_a, phase, g.spin) ? 1 : 0) != 0;   // one verdict for the CTA
     phase ^= 1u;
@@ -206,7 +282,7 @@ __global__ void __launch_bounds__(128) k_gemm(GemmArgs g, int ksplit, float* par
     // 128-byte row segments (8 threads per row, 16-byte accesses); row stride 36 floats keeps
     // both phases free of bank conflicts
     const bool have = kend > kbeg;
-    float* Cs = reinterpret_cast<float*>(smem);
+    float* Cs = reinterpret_cast<float*>(smem + kStageOff);
     const int lrow = warp * 32 + lane;
     for (int h = 0; h < TBN / 32; ++h) {
 #pragma unroll
@@ -239,11 +315,25 @@ __global__ void __launch_bounds__(128) k_gemm(GemmArgs g, int ksplit, float* par
             const float4 c4 = *reinterpret_cast<const float4*>(C);
             o.x += g.beta * c4.x; o.y += g.beta * c4.y; o.z += g.beta * c4.z; o.w += g.beta * c4.w;
           }
+          if (g.bias) {   // z = C + b kept in C, its activation in V (the next layer's input)
+            o.x += g.bias[col]; o.y += g.bias[col + 1]; o.z += g.bias[col + 2]; o.w += g.bias[col + 3];
+            if (g.V) {
+              float4 a = o;
+              if (g.act) a = make_float4(gelu(o.x), gelu(o.y), gelu(o.z), gelu(o.w));
+              *reinterpret_cast<float4*>(g.V + (long long)row * g.ldc + col) = a;
+            }
+          }
           *reinterpret_cast<float4*>(C) = o;
         } else {
           const float vv[4] = {v.x, v.y, v.z, v.w};
-          for (int e = 0; e < 4 && col + e < g.N; ++e)
-            C[e] = g.beta == 0.f ? g.alpha * vv[e] : g.alpha * vv[e] + g.beta * C[e];
+          for (int e = 0; e < 4 && col + e < g.N; ++e) {
+            float o = g.beta == 0.f ? g.alpha * vv[e] : g.alpha * vv[e] + g.beta * C[e];
+            if (g.bias) {
+              o += g.bias[col + e];
+              if (g.V) g.V[(long long)row * g.ldc + col + e] = g.act ? gelu(o) : o;
+            }
+            C[e] = o;
+          }
         }
       }
       __syncthreads();
@@ -272,7 +362,12 @@ __global__ void __launch_bounds__(128) k_gemm(GemmArgs g, int ksplit, float* par
           const float v = __uint_as_float(r[j]);
           if (ksplit == 1) {
             float* C = g.C + (long long)bz * g.sC + (long long)row * g.ldc + col;
-            *C = g.beta == 0.f ? g.alpha * v : g.alpha * v + g.beta * *C;
+            float o = g.beta == 0.f ? g.alpha * v : g.alpha * v + g.beta * *C;
+            if (g.bias) {
+              o += g.bias[col];
+              if (g.V) g.V[(long long)row * g.ldc + col] = g.act ? gelu(o) : o;
+            }
+            *C = o;
           } else {
             partial[(((long long)ks * g.batch + bz) * g.M + row) * g.N + col] = v;
           }
@@ -280,10 +375,271 @@ __global__ void __launch_bounds__(128) k_gemm(GemmArgs g, int ksplit, float* par
       }
     }
   }
+  // accumulator read, operand tiles free for the next row tile
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   if (warp == 0)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
+}
+
+// ---------------------------------------------------------------------------------
+// The products of one transform or mixing step in one launch (BF16 tcgen05.mma as k_gemm, one
+// accumulator per product, so that each sum of two products is rounded as by two k_gemm calls
+// of which the second adds to the first's result):
+//   kPairs     C0 = A0 B0 + s01 A1 B1, C1 = t0 A0 B1 + t1 A1 B0   (complex products)
+//   kTwoLeft   C0 = A0 B0, C1 = A1 B0                             (real data onto two bases)
+//   kSum       C0 = (beta C0 + A0 B0) + A1 B1                     (two bases back to real data)
+// Against a launch per product, each with one 128 x 64 tile per batch item: these products
+// have 8 to 63 rows and 24 or 32 columns an item, and what they cost is the tiles' set-up and the
+// loads of their operands. Here a CTA walks tiles, keeps a shared basis staged, fills a
+// tile's columns from several batch items (g.wcols), stages only the rows that exist, and loads each
+// operand once for all its products.
+// ---------------------------------------------------------------------------------
+constexpr int kPairs = 0, kTwoLeft = 1, kSum = 2;
+struct ProdArgs {
+  const float *A0, *A1, *B0, *B1;
+  float *C0, *C1;
+  int M, N, K, lda, ldb, ldc, ta, tb;
+  long long sA, sB, sC;
+  int batch;
+  float s01, t0, t1, beta;
+  int per;              // batch items in a tile's columns (N <= 64 / per), or 0: one item, N in tiles of 64
+  int mt, nt;           // tiles along M; along N (per = 0) or groups of items
+  long long items;
+  int vecC;
+  long long spin;
+  int slot;
+};
+// accumulators: kPairs 4 x 64 of the 512 tensor-memory columns, two CTAs an SM; the others 2 x 64,
+// four CTAs. The shared-memory requests keep it to that.
+template <int MODE> constexpr int prod_accs() { return MODE == kPairs ? 4 : 2; }
+template <int MODE> constexpr int prod_smem() { return MODE == kPairs ? 78 * 1024 : 52 * 1024; }
+static_assert(2 * (kTileABytes + kTileBBytes) + 32 <= 52 * 1024, "staged operands");
+
+__device__ __forceinline__ void tmem_ld16(uint32_t addr, float* v) {
+  uint32_t r[16];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(addr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]);
+}
+
+template <int MODE>
+__global__ void __launch_bounds__(128) k_prod(ProdArgs g) {
+  constexpr int NACC = prod_accs<MODE>();
+  constexpr int COLS = NACC * TBN;
+  extern __shared__ __align__(1024) unsigned char smem[];
+  unsigned char* sA[2] = {smem, smem + kTileABytes};
+  unsigned char* sB[2] = {smem + 2 * kTileABytes, smem + 2 * kTileABytes + kTileBBytes};
+  uint64_t* mbar = reinterpret_cast<uint64_t*>(smem + 2 * (kTileABytes + kTileBBytes));
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(mbar + 1);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const uint32_t mbar_a = smem_u32(mbar);
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)), "r"(COLS)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  if (tid == 0) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mbar_a) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = *tslot;
+  constexpr uint32_t idesc = mma_idesc(TBM, TBN);
+  uint32_t phase = 0;
+  bool ok = true;
+  int staged_m0 = -1;   // rows of a basis shared by the batch already staged (one K chunk)
+  // where an item's tile lies
+  struct Tile { int b0, n0, m0, cols; };
+  auto tile = [&](long long item) {
+    Tile t;
+    const int mi = (int)(item % g.mt);
+    const long long rest = item / g.mt;
+    const int ni = (int)(rest % g.nt);
+    t.b0 = g.per > 0 ? ni * g.per : (int)(rest / g.nt);
+    t.n0 = g.per > 0 ? 0 : ni * TBN;
+    t.m0 = mi * TBM;
+    t.cols = g.per > 0 ? min(g.per, g.batch - t.b0) * g.N : min(TBN, g.N - t.n0);
+    return t;
+  };
+  // the B operands of a tile's K chunk in registers: every load in flight at once, and those of
+  // the next chunk or item under this one's MMA and epilogue
+  constexpr int NB = TBN * (TBK / 8) / 128, HB = MODE == kTwoLeft ? 1 : 2;
+  float vb[HB][NB][8];
+  auto loadB = [&](const Tile& t, int k0) {
+    const int kn = min(TBK, g.K - k0), kcn = (kn + 15) / 16 * 2;
+#pragma unroll
+    for (int u = 0; u < NB; ++u) {
+      const int c = tid + u * 128;
+      int n, kc;
+      if (g.tb) { n = c / kcn; kc = c - n * kcn; }
+      else { kc = c / TBN; n = c - kc * TBN; }
+      if (kc >= kcn || n >= t.cols) continue;
+      const int j0 = g.per > 0 ? n / g.N : 0;
+      const int gn = g.per > 0 ? n - j0 * g.N : t.n0 + n;
+      const long long off =
+          (long long)(t.b0 + j0) * g.sB + (g.tb ? (long long)gn * g.ldb + k0 : (long long)k0 * g.ldb + gn);
+      const int ks = g.tb ? 1 : g.ldb;
+#pragma unroll
+      for (int h = 0; h < HB; ++h) {
+        const float* B = (h ? g.B1 : g.B0) + off;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) vb[h][u][j] = kc * 8 + j < kn ? B[(long long)(kc * 8 + j) * ks] : 0.f;
+      }
+    }
+  };
+  if (blockIdx.x < g.items) loadB(tile(blockIdx.x), 0);
+  for (long long item = blockIdx.x; item < g.items && ok; item += gridDim.x) {
+    const Tile t = tile(item);
+    const int b0 = t.b0, n0 = t.n0, m0 = t.m0, cols = t.cols;
+    const int rows = min(TBM, g.M - m0), rows8 = (rows + 7) & ~7;
+    const bool keepA = g.sA == 0 && g.K <= TBK;
+    for (int k0 = 0; k0 < g.K && ok; k0 += TBK) {
+      const int kn = min(TBK, g.K - k0);
+      const int kcn = (kn + 15) / 16 * 2;   // 8-element K groups up to the MMA's multiple of 16
+      if (!(keepA && staged_m0 == m0)) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const float* A = (h ? g.A1 : g.A0) + (long long)b0 * g.sA;
+          for (int c = tid; c < rows8 * kcn; c += 128) {
+            int r, kc;
+            if (!g.ta) { r = c / kcn; kc = c - r * kcn; }
+            else { kc = c / rows8; r = c - kc * rows8; }
+            float v[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+              const int k = kc * 8 + j;
+              v[j] = 0.f;
+              if (r < rows && k < kn)
+                v[j] = g.ta ? A[(long long)(k0 + k) * g.lda + m0 + r] : A[(long long)(m0 + r) * g.lda + k0 + k];
+            }
+            *reinterpret_cast<uint4*>(sA[h] + ((kc * (TBM / 8) + (r >> 3)) * 8 + (r & 7)) * 16) =
+                make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
+          }
+        }
+        staged_m0 = keepA ? m0 : -1;
+      }
+      // the tile's columns (columns past `cols` keep what is there: they reach no result)
+#pragma unroll
+      for (int u = 0; u < NB; ++u) {
+        const int c = tid + u * 128;
+        int n, kc;
+        if (g.tb) { n = c / kcn; kc = c - n * kcn; }
+        else { kc = c / TBN; n = c - kc * TBN; }
+        if (kc >= kcn || n >= cols) continue;
+#pragma unroll
+        for (int h = 0; h < HB; ++h) {
+          const float* v = vb[h][u];
+          *reinterpret_cast<uint4*>(sB[h] + ((kc * (TBN / 8) + (n >> 3)) * 8 + (n & 7)) * 16) =
+              make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
+        }
+      }
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      __syncthreads();
+      if (tid == 0) {
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        // accumulators: A0 B0, A1 B1, A0 B1, A1 B0 (kPairs); A0 B0, A1 B0; A0 B0, A1 B1
+#pragma unroll
+        for (int q = 0; q < NACC; ++q) {
+          const int ha = q == 0 || q == 2 ? 0 : 1;
+          const int hb = MODE == kTwoLeft ? 0 : (q == 1 || q == 2 ? 1 : 0);
+          for (int s = 0; s < kcn / 2; ++s) {
+            const uint64_t ad = smem_desc(smem_u32(sA[ha]) + s * 2 * (TBM / 8) * 128, (TBM / 8) * 128, 128);
+            const uint64_t bd = smem_desc(smem_u32(sB[hb]) + s * 2 * (TBN / 8) * 128, (TBN / 8) * 128, 128);
+            const uint32_t acc = (k0 > 0 || s > 0) ? 1u : 0u;
+            asm volatile(
+                "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+                " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem + (uint32_t)(q * TBN)),
+                "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
+                : "memory");
+          }
+        }
+        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar_a)
+                     : "memory");
+      }
+      if (k0 + TBK < g.K) loadB(t, k0 + TBK);
+      else if (item + gridDim.x < g.items) loadB(tile(item + gridDim.x), 0);
+      ok = __syncthreads_and(mbar_wait(mbar_a, phase, g.spin) ? 1 : 0) != 0;   // one verdict for the CTA
+      phase ^= 1u;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    }
+    if (!ok) {
+      // drain: wait (with the default bound) for the committed MMAs before the accumulators are freed
+      if (tid == 0) atomicExch(&g_gemm_timeout[g.slot], 1);
+      mbar_wait(mbar_a, phase ^ 1u);
+      break;
+    }
+    if (warp * 32 < rows) {
+      const int row = m0 + warp * 32 + lane;
+      const bool live = warp * 32 + lane < rows;
+      const uint32_t tw = tmem + ((uint32_t)(warp * 32) << 16);
+      for (int c0 = 0; c0 < cols; c0 += 16) {
+        float p[NACC][16];
+#pragma unroll
+        for (int q = 0; q < NACC; ++q) tmem_ld16(tw + (uint32_t)(q * TBN + c0), p[q]);
+#pragma unroll
+        for (int h = 0; h < (MODE == kSum ? 1 : 2); ++h) {
+          if (!live) break;
+          float o[16];
+#pragma unroll
+          for (int j = 0; j < 16; ++j)
+            o[j] = MODE == kPairs ? (h ? g.t0 * p[2][j] + g.t1 * p[NACC - 1][j] : p[0][j] + g.s01 * p[1][j])
+                                  : (MODE == kTwoLeft ? p[h][j] : p[0][j]);
+          float* C = h ? g.C1 : g.C0;
+#pragma unroll
+          for (int j4 = 0; j4 < 16; j4 += 4) {
+            const int n = c0 + j4;
+            if (n >= cols) break;
+            const int j0 = g.per > 0 ? n / g.N : 0;
+            float* d = C + (long long)(b0 + j0) * g.sC + (long long)row * g.ldc + (g.per > 0 ? n - j0 * g.N : n0 + n);
+            if (g.vecC) {   // N, the strides and the base are multiples of four floats
+              float4 w = make_float4(o[j4], o[j4 + 1], o[j4 + 2], o[j4 + 3]);
+              if (MODE == kSum) {
+                if (g.beta != 0.f) {
+                  const float4 c4 = *reinterpret_cast<const float4*>(d);
+                  w.x += c4.x; w.y += c4.y; w.z += c4.z; w.w += c4.w;
+                }
+                w.x += p[1][j4]; w.y += p[1][j4 + 1]; w.z += p[1][j4 + 2]; w.w += p[1][j4 + 3];
+              }
+              *reinterpret_cast<float4*>(d) = w;
+            } else {
+              for (int e = 0; e < 4 && n + e < cols; ++e) {
+                const int je = g.per > 0 ? (n + e) / g.N : 0;
+                float* de = C + (long long)(b0 + je) * g.sC + (long long)row * g.ldc +
+                            (g.per > 0 ? n + e - je * g.N : n0 + n + e);
+                float w = o[j4 + e];
+                if (MODE == kSum) {
+                  if (g.beta != 0.f) w += *de;
+                  w += p[1][j4 + e];
+                }
+                *de = w;
+              }
+            }
+          }
+        }
+        __syncwarp();   // the next accumulator reads are for the whole warp
+      }
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();   // accumulators read, operand tiles free
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (warp == 0)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(COLS) : "memory");
 }
 
 __global__ void k_gemm_reduce(GemmArgs g, int ksplit, const float* partial) {
@@ -327,6 +683,16 @@ cudaError_t gemm_timeout_read(int slot, int* host_flag, cudaStream_t s) {
 static thread_local float* g_split_ws = nullptr;
 static thread_local long long g_split_floats = 0;
 
+static void launch_gemm(const GemmArgs& g, int gm, int gn, int ksplit, cudaStream_t s) {
+  if (g.K <= TBK) {
+    const long long others = (long long)gn * g.batch * ksplit;
+    const int gy = (int)std::max<long long>(1, std::min<long long>(gm, 152 * 8 / others));
+    k_gemm<false><<<dim3(gn, gy, g.batch * ksplit), 128, kGemmSmem, s>>>(g, ksplit, g_split_ws);
+  } else {
+    k_gemm<true><<<dim3(gn, gm, g.batch * ksplit), 128, kGemmSmem, s>>>(g, ksplit, g_split_ws);
+  }
+}
+
 cudaError_t gemm_bf16(const GemmArgs& g0, cudaStream_t s) {
   if (g0.M <= 0 || g0.N <= 0 || g0.batch <= 0) return cudaSuccess;
   GemmArgs g = g0;
@@ -334,7 +700,7 @@ cudaError_t gemm_bf16(const GemmArgs& g0, cudaStream_t s) {
   g.spin = g_ctx_spin > 0 ? g_ctx_spin : kMbarSpinLimit;
   auto al16 = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
   g.vecA = !g.ta && g.lda % 4 == 0 && g.sA % 4 == 0 && al16(g.A);
-  g.vecC = g.ldc % 4 == 0 && g.sC % 4 == 0 && al16(g.C);
+  g.vecC = g.ldc % 4 == 0 && g.sC % 4 == 0 && al16(g.C) && (g.V == nullptr || al16(g.V));
   if ((g.M + TBM - 1) / TBM > 65535) {   // grid y is limited to 65535 tiles: chunks of rows
     const int rows = 65535 * TBM;
     for (int r0 = 0; r0 < g.M; r0 += rows) {
@@ -342,6 +708,7 @@ cudaError_t gemm_bf16(const GemmArgs& g0, cudaStream_t s) {
       h.M = std::min(rows, g.M - r0);
       h.A = g.ta ? g.A + r0 : g.A + (long long)r0 * g.lda;
       h.C = g.C + (long long)r0 * g.ldc;
+      if (g.V) h.V = g.V + (long long)r0 * g.ldc;
       const cudaError_t e = gemm_bf16(h, s);
       if (e != cudaSuccess) return e;
     }
@@ -350,7 +717,7 @@ cudaError_t gemm_bf16(const GemmArgs& g0, cudaStream_t s) {
   const int gm = (g.M + TBM - 1) / TBM, gn = (g.N + TBN - 1) / TBN;
   int ksplit = 1;
   const long long tiles = (long long)gm * gn * g.batch;
-  if (tiles < 152 && g.K > 2048 && g_split_ws) {
+  if (tiles < 152 && g.K > 2048 && g_split_ws && !g.bias) {
     ksplit = (int)std::min<long long>(256, std::max<long long>(1, (304 + tiles - 1) / tiles));
     ksplit = std::min(ksplit, (g.K + 1023) / 1024);
     while (ksplit > 1 && (long long)ksplit * g.M * g.N * g.batch > g_split_floats) --ksplit;
@@ -362,12 +729,11 @@ cudaError_t gemm_bf16(const GemmArgs& g0, cudaStream_t s) {
       h.A = g.A + (long long)b0 * g.sA;
       h.B = g.B + (long long)b0 * g.sB;
       h.C = g.C + (long long)b0 * g.sC;
-      k_gemm<<<dim3(gn, gm, h.batch), 128, kGemmSmem, s>>>(h, 1, nullptr);
+      launch_gemm(h, gm, gn, 1, s);
     }
     return cudaGetLastError();
   }
-  dim3 grid(gn, gm, g.batch * ksplit);
-  k_gemm<<<grid, 128, kGemmSmem, s>>>(g, ksplit, g_split_ws);
+  launch_gemm(g, gm, gn, ksplit, s);
   if (ksplit > 1) {
     const long long total = (long long)g.M * g.N * g.batch;
     const int blocks = (int)std::min<long long>((total + 255) / 256, 152 * 8);
@@ -379,19 +745,8 @@ cudaError_t gemm_bf16(const GemmArgs& g0, cudaStream_t s) {
 // ---------------------------------------------------------------------------------
 // elementwise kernels
 // ---------------------------------------------------------------------------------
-__device__ __forceinline__ float gelu(float x) { return 0.5f * x * (1.f + erff(x * 0.70710678118654752f)); }
 __device__ __forceinline__ float gelu_d(float x) {
   return 0.5f * (1.f + erff(x * 0.70710678118654752f)) + x * 0.39894228040143268f * expf(-0.5f * x * x);
-}
-
-// z += b (per column); v = act(z)
-__global__ void k_bias_act(float* z, const float* b, float* v, long long rows, int cols, int act) {
-  const long long n = rows * cols;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const float t = z[i] + b[i % cols];
-    z[i] = t;
-    v[i] = act ? gelu(t) : t;
-  }
 }
 
 __global__ void k_gelu_back(const float* dv, const float* z, float* dz, long long n) {
@@ -399,22 +754,50 @@ __global__ void k_gelu_back(const float* dv, const float* z, float* dz, long lon
     dz[i] = dv[i] * gelu_d(z[i]);
 }
 
-// deterministic column sums: stage 1 per row block, stage 2 over blocks
-__global__ void k_colsum1(const float* x, long long rows, int cols, int rows_per, float* part) {
-  const long long r0 = (long long)blockIdx.x * rows_per;
-  const long long r1 = min(rows, r0 + rows_per);
-  for (int c = threadIdx.x; c < cols; c += blockDim.x) {
-    float s = 0.f;
-    for (long long r = r0; r < r1; ++r) s += x[r * cols + c];
-    part[(long long)blockIdx.x * cols + c] = s;
+// deterministic column sums: stage 1 per row block, stage 2 over the blocks, each column added in
+// order by one thread from rows that the whole CTA has staged (the additions are a chain of
+// short latencies; straight from global memory it was a chain of long ones: 33 and 41 us, now 7
+// and 4 us for 127008 rows of 32 columns)
+constexpr int kColRows = 64, kColMax = 128;
+__device__ __forceinline__ void colsum_staged(const float* x, long long r0, long long r1, int cols, int c0, float* tile,
+                                              float* out) {
+  const int nc = min(kColMax, cols - c0);
+  float s = 0.f;
+  for (long long r = r0; r < r1; r += kColRows) {
+    const int n = (int)min((long long)kColRows, r1 - r);
+    for (int t0 = threadIdx.x; t0 < n * nc; t0 += 8 * blockDim.x) {   // eight loads in flight a thread
+      float v[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int t = t0 + u * (int)blockDim.x, i = t / nc;
+        if (t < n * nc) v[u] = x[(r + i) * cols + c0 + t - i * nc];
+      }
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int t = t0 + u * (int)blockDim.x, i = t / nc;
+        if (t < n * nc) tile[i * kColMax + t - i * nc] = v[u];
+      }
+    }
+    __syncthreads();
+    if (threadIdx.x < nc) {
+#pragma unroll 16
+      for (int i = 0; i < n; ++i) s += tile[i * kColMax + threadIdx.x];
+    }
+    __syncthreads();
   }
+  if (threadIdx.x < nc) out[c0 + threadIdx.x] = s;
 }
-__global__ void k_colsum2(const float* part, int nblk, int cols, float* out) {
-  for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < cols; c += gridDim.x * blockDim.x) {
-    float s = 0.f;
-    for (int b = 0; b < nblk; ++b) s += part[(long long)b * cols + c];
-    out[c] = s;
-  }
+__global__ void __launch_bounds__(256) k_colsum1(const float* x, long long rows, int cols, int rows_per, float* part) {
+  __shared__ float tile[kColRows * kColMax];
+  const long long r0 = min(rows, (long long)blockIdx.x * rows_per);
+  const long long r1 = min(rows, r0 + rows_per);
+  for (int c0 = 0; c0 < cols; c0 += kColMax)
+    colsum_staged(x, r0, r1, cols, c0, tile, part + (long long)blockIdx.x * cols);
+}
+__global__ void __launch_bounds__(256) k_colsum2(const float* part, int nblk, int cols, float* out) {
+  __shared__ float tile[kColRows * kColMax];
+  for (int c0 = blockIdx.x * kColMax; c0 < cols; c0 += gridDim.x * kColMax)
+    colsum_staged(part, 0, nblk, cols, c0, tile, out);
 }
 
 __global__ void k_mse(const float* out, const float* t, float* dout, long long n, float* part) {
@@ -436,11 +819,10 @@ __global__ void k_mse(const float* out, const float* t, float* dout, long long n
   }
 }
 __global__ void k_mse_final(const float* part, int nblk, long long n, float* loss) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    double s = 0.0;
-    for (int b = 0; b < nblk; ++b) s += part[b];
-    *loss = (float)(s / (double)n);
-  }
+  double s = 0.0;
+  for (int b = threadIdx.x; b < nblk; b += 32) s += part[b];
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+  if (threadIdx.x == 0) *loss = (float)(s / (double)n);
 }
 
 __global__ void k_adam(float* p, const float* g, float* m, float* v, long long n, float lr, float b1, float b2,
@@ -604,6 +986,46 @@ static GemmArgs gemm(const float* A, const float* B, float* C, int M, int N, int
   GemmArgs g;
   g.A = A; g.B = B; g.C = C; g.M = M; g.N = N; g.K = K; g.lda = lda; g.ldb = ldb; g.ldc = ldc;
   g.ta = ta; g.tb = tb; g.sA = sA; g.sB = sB; g.sC = sC; g.batch = batch; g.alpha = alpha; g.beta = beta;
+  g.bias = nullptr; g.V = nullptr; g.act = 0;
+  return g;
+}
+
+static ProdArgs prod(const float* A0, const float* A1, const float* B0, const float* B1, float* C0, float* C1, int M,
+                     int N, int K, int lda, int ldb, int ldc, int ta, int tb, long long sA, long long sB, long long sC,
+                     int batch) {
+  ProdArgs g{};
+  g.A0 = A0; g.A1 = A1; g.B0 = B0; g.B1 = B1; g.C0 = C0; g.C1 = C1; g.M = M; g.N = N; g.K = K;
+  g.lda = lda; g.ldb = ldb; g.ldc = ldc; g.ta = ta; g.tb = tb; g.sA = sA; g.sB = sB; g.sC = sC; g.batch = batch;
+  return g;
+}
+
+template <int MODE> static cudaError_t run_prod(ProdArgs g, cudaStream_t s) {
+  if (g.M <= 0 || g.N <= 0 || g.batch <= 0) return cudaSuccess;
+  auto al16 = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
+  g.slot = g_ctx_slot;
+  g.spin = g_ctx_spin > 0 ? g_ctx_spin : kMbarSpinLimit;
+  // several items side by side where they share A and two or more fit in a tile
+  g.per = g.sA == 0 && 2 * g.N <= TBN && g.batch > 1 ? TBN / g.N : 0;
+  g.vecC = g.N % 4 == 0 && g.ldc % 4 == 0 && g.sC % 4 == 0 && al16(g.C0) && (MODE == kSum || al16(g.C1));
+  g.mt = (g.M + TBM - 1) / TBM;
+  g.nt = g.per > 0 ? (g.batch + g.per - 1) / g.per : (g.N + TBN - 1) / TBN;
+  g.items = (long long)g.mt * g.nt * (g.per > 0 ? 1 : g.batch);
+  static std::atomic<int> cache[kAttrDevices] = {};
+  const cudaError_t e = smem_attr(k_prod<MODE>, prod_smem<MODE>(), cache);
+  if (e != cudaSuccess) return e;
+  const long long grid = std::min<long long>(g.items, 152LL * (MODE == kPairs ? 2 : 4));
+  k_prod<MODE><<<(int)grid, 128, prod_smem<MODE>(), s>>>(g);
+  return cudaGetLastError();
+}
+// C0 = A0 B0 + s01 A1 B1, C1 = t0 A0 B1 + t1 A1 B0
+static cudaError_t prod_pairs(ProdArgs g, float s01, float t0, float t1, cudaStream_t s) {
+  g.s01 = s01; g.t0 = t0; g.t1 = t1;
+  return run_prod<kPairs>(g, s);
+}
+
+// C = A B (+ C) + bias with the activation of the sum in V (NULL: C is the result itself)
+static GemmArgs with_bias(GemmArgs g, const float* bias, float* V, int act) {
+  g.bias = bias; g.V = V; g.act = act;
   return g;
 }
 
@@ -616,8 +1038,8 @@ static GemmArgs gemm(const float* A, const float* B, float* C, int M, int N, int
 static cudaError_t colsum(const float* x, long long rows, int cols, float* out, float* part, cudaStream_t s) {
   const int nblk = (int)std::min<long long>(1024, std::max<long long>(1, rows / 256));
   const int rows_per = (int)((rows + nblk - 1) / nblk);
-  k_colsum1<<<nblk, 128, 0, s>>>(x, rows, cols, rows_per, part);
-  k_colsum2<<<(cols + 127) / 128, 128, 0, s>>>(part, nblk, cols, out);
+  k_colsum1<<<nblk, 256, 0, s>>>(x, rows, cols, rows_per, part);
+  k_colsum2<<<(cols + kColMax - 1) / kColMax, 256, 0, s>>>(part, nblk, cols, out);
   return cudaGetLastError();
 }
 
@@ -635,7 +1057,7 @@ static Bases bases_of(const NetConfig& c, const float* b) {
   return r;
 }
 
-// Complex DFT along one axis on the kept modes, as four real GEMMs per batch item, with
+// Complex DFT along one axis on the kept modes, as four real products per batch item, with
 // bases Gc, Gs [K1 x Nn] and Hc, Hs [Nn x K1]; C columns per row, batch strides in floats.
 //   forward  O = G I:  Or = Gc Ir + Gs Ii,  Oi = Gc Ii - Gs Ir   (e^{-2 pi i k y / N})
 //   inverse  O = H I:  Or = Hc Ir - Hs Ii,  Oi = Hc Ii + Hs Ir   (e^{+2 pi i k y / N})
@@ -645,32 +1067,22 @@ struct Axis {
   cudaStream_t s;
   cudaError_t fwd(const float* ir, const float* ii, float* orr, float* oi, int C, long long sI, long long sO,
                   int batch) const {
-    NCK(gemm_bf16(gemm(bs.Gc, ir, orr, K1, C, Nn, Nn, C, C, 0, 0, 0, sI, sO, batch, 1.f, 0.f), s));
-    NCK(gemm_bf16(gemm(bs.Gs, ii, orr, K1, C, Nn, Nn, C, C, 0, 0, 0, sI, sO, batch, 1.f, 1.f), s));
-    NCK(gemm_bf16(gemm(bs.Gc, ii, oi, K1, C, Nn, Nn, C, C, 0, 0, 0, sI, sO, batch, 1.f, 0.f), s));
-    return gemm_bf16(gemm(bs.Gs, ir, oi, K1, C, Nn, Nn, C, C, 0, 0, 0, sI, sO, batch, -1.f, 1.f), s);
+    return prod_pairs(prod(bs.Gc, bs.Gs, ir, ii, orr, oi, K1, C, Nn, Nn, C, C, 0, 0, 0, sI, sO, batch), 1.f, 1.f, -1.f, s);
   }
   cudaError_t inv(const float* ir, const float* ii, float* orr, float* oi, int C, long long sI, long long sO,
                   int batch) const {
-    NCK(gemm_bf16(gemm(bs.Hc, ir, orr, Nn, C, K1, K1, C, C, 0, 0, 0, sI, sO, batch, 1.f, 0.f), s));
-    NCK(gemm_bf16(gemm(bs.Hs, ii, orr, Nn, C, K1, K1, C, C, 0, 0, 0, sI, sO, batch, -1.f, 1.f), s));
-    NCK(gemm_bf16(gemm(bs.Hc, ii, oi, Nn, C, K1, K1, C, C, 0, 0, 0, sI, sO, batch, 1.f, 0.f), s));
-    return gemm_bf16(gemm(bs.Hs, ir, oi, Nn, C, K1, K1, C, C, 0, 0, 0, sI, sO, batch, 1.f, 1.f), s);
+    return prod_pairs(prod(bs.Hc, bs.Hs, ir, ii, orr, oi, Nn, C, K1, K1, C, C, 0, 0, 0, sI, sO, batch), -1.f, 1.f, 1.f, s);
   }
   // adjoints: dI = G^T dO (of fwd), dI = H^T dO (of inv); dO has stride sO, dI stride sI
   cudaError_t fwd_adj(const float* dor, const float* doi, float* dir, float* dii, int C, long long sO,
                       long long sI, int batch) const {
-    NCK(gemm_bf16(gemm(bs.Gc, dor, dir, Nn, C, K1, Nn, C, C, 1, 0, 0, sO, sI, batch, 1.f, 0.f), s));
-    NCK(gemm_bf16(gemm(bs.Gs, doi, dir, Nn, C, K1, Nn, C, C, 1, 0, 0, sO, sI, batch, -1.f, 1.f), s));
-    NCK(gemm_bf16(gemm(bs.Gs, dor, dii, Nn, C, K1, Nn, C, C, 1, 0, 0, sO, sI, batch, 1.f, 0.f), s));
-    return gemm_bf16(gemm(bs.Gc, doi, dii, Nn, C, K1, Nn, C, C, 1, 0, 0, sO, sI, batch, 1.f, 1.f), s);
+    return prod_pairs(prod(bs.Gc, bs.Gs, dor, doi, dir, dii, Nn, C, K1, Nn, C, C, 1, 0, 0, sO, sI, batch), -1.f, 1.f, 1.f,
+                      s);
   }
   cudaError_t inv_adj(const float* dor, const float* doi, float* dir, float* dii, int C, long long sO,
                       long long sI, int batch) const {
-    NCK(gemm_bf16(gemm(bs.Hc, dor, dir, K1, C, Nn, K1, C, C, 1, 0, 0, sO, sI, batch, 1.f, 0.f), s));
-    NCK(gemm_bf16(gemm(bs.Hs, doi, dir, K1, C, Nn, K1, C, C, 1, 0, 0, sO, sI, batch, 1.f, 1.f), s));
-    NCK(gemm_bf16(gemm(bs.Hc, doi, dii, K1, C, Nn, K1, C, C, 1, 0, 0, sO, sI, batch, 1.f, 0.f), s));
-    return gemm_bf16(gemm(bs.Hs, dor, dii, K1, C, Nn, K1, C, C, 1, 0, 0, sO, sI, batch, -1.f, 1.f), s);
+    return prod_pairs(prod(bs.Hc, bs.Hs, dor, doi, dir, dii, K1, C, Nn, K1, C, C, 1, 0, 0, sO, sI, batch), 1.f, 1.f, -1.f,
+                      s);
   }
 };
 
@@ -689,15 +1101,15 @@ cudaError_t net_forward(const NetConfig& c, const float* prm, const float* bases
   const int BN = (int)(B * ipow(N, d - 1));   // rows of x transforms: (b, (z,) y)
   const long long nmodes = spectral_modes(c);
   // lift
-  NCK(gemm_bf16(gemm(in, prm + o.lift_w, w.v[0], (int)P, W, c.cin, c.cin, W, W, 0, 0, 0, 0, 0, 1, 1.f, 0.f), s));
-  k_bias_act<<<eblocks(P * W), 256, 0, s>>>(w.v[0], prm + o.lift_b, w.v[0], P, W, 0);
+  NCK(gemm_bf16(with_bias(gemm(in, prm + o.lift_w, w.v[0], (int)P, W, c.cin, c.cin, W, W, 0, 0, 0, 0, 0, 1, 1.f, 0.f),
+                          prm + o.lift_b, nullptr, 0), s));
   for (int l = 0; l < c.layers; ++l) {
     const float* v = w.v[l];
     const float* Rr = prm + o.R[l];
     const float* Ri = Rr + nmodes * W * W;
     // (1) x DFT, per (b, (z,) y): [K x N] x [N x W]
-    NCK(gemm_bf16(gemm(bs.Fr, v, w.x1r, K, W, N, N, W, W, 0, 0, 0, (long long)N * W, (long long)K * W, BN, 1.f, 0.f), s));
-    NCK(gemm_bf16(gemm(bs.Fi, v, w.x1i, K, W, N, N, W, W, 0, 0, 0, (long long)N * W, (long long)K * W, BN, 1.f, 0.f), s));
+    NCK(run_prod<kTwoLeft>(prod(bs.Fr, bs.Fi, v, nullptr, w.x1r, w.x1i, K, W, N, N, W, W, 0, 0, 0, (long long)N * W,
+                                (long long)K * W, BN), s));
     // (2) y DFT per (b, (z)): [K1 x N] x [N x KW]; (2z) z DFT per b: [K1 x N] x [N x K1 KW]
     const long long sx1 = (long long)N * KW, sx2 = (long long)K1 * KW;
     if (d == 2) {
@@ -709,10 +1121,8 @@ cudaError_t net_forward(const NetConfig& c, const float* prm, const float* bases
     // (3) per mode m: Y = X2 R (complex), rows b (stride nmodes*W), batch over modes
     const int nm = (int)nmodes;
     const int ldm = nm * W;
-    NCK(gemm_bf16(gemm(w.x2r[l], Rr, w.yr, B, W, W, ldm, W, ldm, 0, 0, W, (long long)W * W, W, nm, 1.f, 0.f), s));
-    NCK(gemm_bf16(gemm(w.x2i[l], Ri, w.yr, B, W, W, ldm, W, ldm, 0, 0, W, (long long)W * W, W, nm, -1.f, 1.f), s));
-    NCK(gemm_bf16(gemm(w.x2r[l], Ri, w.yi, B, W, W, ldm, W, ldm, 0, 0, W, (long long)W * W, W, nm, 1.f, 0.f), s));
-    NCK(gemm_bf16(gemm(w.x2i[l], Rr, w.yi, B, W, W, ldm, W, ldm, 0, 0, W, (long long)W * W, W, nm, 1.f, 1.f), s));
+    NCK(prod_pairs(prod(w.x2r[l], w.x2i[l], Rr, Ri, w.yr, w.yi, B, W, W, ldm, W, ldm, 0, 0, W, (long long)W * W, W, nm),
+                   -1.f, 1.f, 1.f, s));
     // (4) inverse (z then) y
     if (d == 2) {
       NCK(ax.inv(w.yr, w.yi, w.z1r, w.z1i, KW, sx2, sx1, B));
@@ -721,17 +1131,17 @@ cudaError_t net_forward(const NetConfig& c, const float* prm, const float* bases
       NCK(ax.inv(w.mr, w.mi, w.z1r, w.z1i, KW, sx2, sx1, B * N));
     }
     // (5) inverse x (half spectrum), per (b, (z,) y): s = Er Z1r + Ei Z1i   ([N x K] x [K x W]) into z
-    NCK(gemm_bf16(gemm(bs.Er, w.z1r, w.z[l], N, W, K, K, W, W, 0, 0, 0, (long long)K * W, (long long)N * W, BN, 1.f, 0.f), s));
-    NCK(gemm_bf16(gemm(bs.Ei, w.z1i, w.z[l], N, W, K, K, W, W, 0, 0, 0, (long long)K * W, (long long)N * W, BN, 1.f, 1.f), s));
+    NCK(run_prod<kSum>(prod(bs.Er, bs.Ei, w.z1r, w.z1i, w.z[l], nullptr, N, W, K, K, W, W, 0, 0, 0, (long long)K * W,
+                            (long long)N * W, BN), s));
     // (6) z += v W ; (7) bias + activation
-    NCK(gemm_bf16(gemm(v, prm + o.W[l], w.z[l], (int)P, W, W, W, W, W, 0, 0, 0, 0, 0, 1, 1.f, 1.f), s));
-    k_bias_act<<<eblocks(P * W), 256, 0, s>>>(w.z[l], prm + o.b[l], w.v[l + 1], P, W, l + 1 < c.layers ? 1 : 0);
+    NCK(gemm_bf16(with_bias(gemm(v, prm + o.W[l], w.z[l], (int)P, W, W, W, W, W, 0, 0, 0, 0, 0, 1, 1.f, 1.f),
+                            prm + o.b[l], w.v[l + 1], l + 1 < c.layers ? 1 : 0), s));
   }
   // projection
-  NCK(gemm_bf16(gemm(w.v[c.layers], prm + o.p1_w, w.pz, (int)P, c.proj, W, W, c.proj, c.proj, 0, 0, 0, 0, 0, 1, 1.f, 0.f), s));
-  k_bias_act<<<eblocks(P * c.proj), 256, 0, s>>>(w.pz, prm + o.p1_b, w.ph, P, c.proj, 1);
-  NCK(gemm_bf16(gemm(w.ph, prm + o.p2_w, out, (int)P, c.cout, c.proj, c.proj, c.cout, c.cout, 0, 0, 0, 0, 0, 1, 1.f, 0.f), s));
-  k_bias_act<<<eblocks(P * c.cout), 256, 0, s>>>(out, prm + o.p2_b, out, P, c.cout, 0);
+  NCK(gemm_bf16(with_bias(gemm(w.v[c.layers], prm + o.p1_w, w.pz, (int)P, c.proj, W, W, c.proj, c.proj, 0, 0, 0, 0, 0, 1,
+                               1.f, 0.f), prm + o.p1_b, w.ph, 1), s));
+  NCK(gemm_bf16(with_bias(gemm(w.ph, prm + o.p2_w, out, (int)P, c.cout, c.proj, c.proj, c.cout, c.cout, 0, 0, 0, 0, 0, 1,
+                               1.f, 0.f), prm + o.p2_b, nullptr, 0), s));
   g_split_ws = nullptr;
   g_split_floats = 0;
   return cudaGetLastError();
@@ -781,8 +1191,8 @@ cudaError_t net_backward(const NetConfig& c, const float* prm, const float* base
     NCK(gemm_bf16(gemm(v, w.dz, grad + o.W[l], W, W, (int)P, W, W, W, 1, 0, 0, 0, 0, 1, 1.f, 0.f), s));
     NCK(gemm_bf16(gemm(w.dz, prm + o.W[l], w.dv, (int)P, W, W, W, W, W, 0, 1, 0, 0, 0, 1, 1.f, 0.f), s));
     // (5') dZ1 = E^T dz, per (b, (z,) y): [K x N] x [N x W]
-    NCK(gemm_bf16(gemm(bs.Er, w.dz, w.dz1r, K, W, N, K, W, W, 1, 0, 0, (long long)N * W, (long long)K * W, BN, 1.f, 0.f), s));
-    NCK(gemm_bf16(gemm(bs.Ei, w.dz, w.dz1i, K, W, N, K, W, W, 1, 0, 0, (long long)N * W, (long long)K * W, BN, 1.f, 0.f), s));
+    NCK(run_prod<kTwoLeft>(prod(bs.Er, bs.Ei, w.dz, nullptr, w.dz1r, w.dz1i, K, W, N, K, W, W, 1, 0, 0, (long long)N * W,
+                                (long long)K * W, BN), s));
     // (4') adjoint of the inverse y (and then z) transform: dY = H^T dZ1
     const long long sx1 = (long long)N * KW, sx2 = (long long)K1 * KW;
     if (d == 2) {
@@ -795,15 +1205,11 @@ cudaError_t net_backward(const NetConfig& c, const float* prm, const float* base
     const int nm = (int)nmodes;
     const int ldm = nm * W;
     const long long WW = (long long)W * W;
-    NCK(gemm_bf16(gemm(w.x2r[l], w.dyr, dRr, W, W, B, ldm, ldm, W, 1, 0, W, W, WW, nm, 1.f, 0.f), s));
-    NCK(gemm_bf16(gemm(w.x2i[l], w.dyi, dRr, W, W, B, ldm, ldm, W, 1, 0, W, W, WW, nm, 1.f, 1.f), s));
-    NCK(gemm_bf16(gemm(w.x2r[l], w.dyi, dRi, W, W, B, ldm, ldm, W, 1, 0, W, W, WW, nm, 1.f, 0.f), s));
-    NCK(gemm_bf16(gemm(w.x2i[l], w.dyr, dRi, W, W, B, ldm, ldm, W, 1, 0, W, W, WW, nm, -1.f, 1.f), s));
+    NCK(prod_pairs(prod(w.x2r[l], w.x2i[l], w.dyr, w.dyi, dRr, dRi, W, W, B, ldm, ldm, W, 1, 0, W, W, WW, nm), 1.f, 1.f,
+                   -1.f, s));
     //      dX2r = dYr Rr^T + dYi Ri^T ; dX2i = dYi Rr^T - dYr Ri^T   ([B x W] x [W x W]^T)
-    NCK(gemm_bf16(gemm(w.dyr, Rr, w.dx2r, B, W, W, ldm, W, ldm, 0, 1, W, WW, W, nm, 1.f, 0.f), s));
-    NCK(gemm_bf16(gemm(w.dyi, Ri, w.dx2r, B, W, W, ldm, W, ldm, 0, 1, W, WW, W, nm, 1.f, 1.f), s));
-    NCK(gemm_bf16(gemm(w.dyi, Rr, w.dx2i, B, W, W, ldm, W, ldm, 0, 1, W, WW, W, nm, 1.f, 0.f), s));
-    NCK(gemm_bf16(gemm(w.dyr, Ri, w.dx2i, B, W, W, ldm, W, ldm, 0, 1, W, WW, W, nm, -1.f, 1.f), s));
+    NCK(prod_pairs(prod(w.dyr, w.dyi, Rr, Ri, w.dx2r, w.dx2i, B, W, W, ldm, W, ldm, 0, 1, W, WW, W, nm), 1.f, -1.f, 1.f,
+                   s));
     // (2') adjoint of the forward (z then) y transform: dX1 = G^T dX2
     if (d == 2) {
       NCK(ax.fwd_adj(w.dx2r, w.dx2i, w.dx1r, w.dx1i, KW, sx2, sx1, B));
@@ -812,8 +1218,10 @@ cudaError_t net_backward(const NetConfig& c, const float* prm, const float* base
       NCK(ax.fwd_adj(w.dmr, w.dmi, w.dx1r, w.dx1i, KW, sx2, sx1, B * N));
     }
     // (1') dv += Fr^T dX1r + Fi^T dX1i, per (b, (z,) y): [N x K] x [K x W]
-    NCK(gemm_bf16(gemm(bs.Fr, w.dx1r, w.dv, N, W, K, N, W, W, 1, 0, 0, (long long)K * W, (long long)N * W, BN, 1.f, 1.f), s));
-    NCK(gemm_bf16(gemm(bs.Fi, w.dx1i, w.dv, N, W, K, N, W, W, 1, 0, 0, (long long)K * W, (long long)N * W, BN, 1.f, 1.f), s));
+    ProdArgs dv = prod(bs.Fr, bs.Fi, w.dx1r, w.dx1i, w.dv, nullptr, N, W, K, N, W, W, 1, 0, 0, (long long)K * W,
+                       (long long)N * W, BN);
+    dv.beta = 1.f;
+    NCK(run_prod<kSum>(dv, s));
   }
   // lift
   NCK(colsum(w.dv, P, W, grad + o.lift_b, w.colpart, s));

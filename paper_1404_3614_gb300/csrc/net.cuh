@@ -45,6 +45,9 @@ struct GemmArgs {
   int vecA, vecC;         // set by gemm_bf16: 16-byte vector loads of A rows / stores of C rows
   long long spin;         // set by gemm_bf16: polls of the completion barrier before giving up
   int slot;               // set by gemm_bf16: the calling context's timeout flag
+  const float* bias = nullptr;   // per column, added to C; then V (leading dimension ldc), if given,
+  float* V = nullptr;            // takes its activation (act: GELU, else the sum itself)
+  int act = 0;
 };
 cudaError_t gemm_bf16(const GemmArgs& g, cudaStream_t s);
 // Number of per-context GEMM timeout flags; context k uses flag k mod kGemmFlagSlots.
