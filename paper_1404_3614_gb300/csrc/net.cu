@@ -20,6 +20,7 @@
 #include <vector>
 
 #include "attr.cuh"
+#include "common.cuh"
 #include "net.cuh"
 
 namespace homb {
@@ -386,6 +387,146 @@ __global__ void __launch_bounds__(128, PIPE ? 3 : 8) k_gemm(GemmArgs g, int kspl
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
 }
 
+__device__ __forceinline__ void tmem_ld16(uint32_t addr, float* v) {
+  uint32_t r[16];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(addr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]);
+}
+
+// Split-K partials of C = A^T B, A [K x M] and B [K x N] row-major (the weight gradients: K the
+// batch's grid points, M and N channels): the same chunks, products and partials as k_gemm, with
+// the FP32 rows of the next chunks copied to shared memory by cp.async, kTnStages chunks deep,
+// while this chunk's are rounded, transposed into the operand tiles and multiplied. A split
+// walks its chunks one after another: with each chunk's loads waited for, 125 splits of 16 chunks
+// (K = 127008, 32 x 32) took 123 us, 71 us with one chunk ahead in registers, 30 us so.
+constexpr int kTnStages = 4;
+__host__ __device__ inline size_t tn_smem(int rows, int cols) {
+  return kTileABytes + kTileBBytes + 16 + (size_t)kTnStages * TBK * (rows + cols) * 4;
+}
+__global__ void __launch_bounds__(256) k_gemm_tn(GemmArgs g, int ksplit, float* partial) {
+  extern __shared__ __align__(1024) unsigned char smem[];
+  unsigned char* sA = smem;
+  unsigned char* sB = smem + kTileABytes;
+  uint64_t* mbar = reinterpret_cast<uint64_t*>(smem + kTileABytes + kTileBBytes);
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(mbar + 1);
+  float* stage = reinterpret_cast<float*>(smem + kTileABytes + kTileBBytes + 16);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int ks = blockIdx.z, n0 = blockIdx.x * TBN, m0 = blockIdx.y * TBM;
+  const int rows = min(TBM, g.M - m0), cols = min(TBN, g.N - n0);   // multiples of four
+  const int kchunk = ((g.K + ksplit - 1) / ksplit + TBK - 1) / TBK * TBK;
+  const int kbeg = ks * kchunk, kend = min(g.K, kbeg + kchunk);
+  const uint32_t mbar_a = smem_u32(mbar);
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)),
+                 "r"(kTmemCols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  if (tid == 0) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mbar_a) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = *tslot;
+  constexpr uint32_t idesc = mma_idesc(TBM, TBN);
+  const int ra = rows / 4, rb = cols / 4, per = ra + rb;   // 16-byte pieces of a staged row: A's, then B's
+  const FastDiv fper((uint32_t)per);
+  auto copy = [&](int k0, int st) {   // chunk k0's rows; rows past kend are not read from shared memory
+    const int kn = min(TBK, kend - k0);
+    float* dst = stage + (size_t)st * TBK * (rows + cols);
+    for (int t = tid; t < kn * per; t += 256) {
+      const int k = fper.div(t), c = t - k * per;
+      const float* src = c < ra ? g.A + (long long)(k0 + k) * g.lda + m0 + 4 * c
+                                : g.B + (long long)(k0 + k) * g.ldb + n0 + 4 * (c - ra);
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_u32(dst + k * (rows + cols) + 4 * c)), "l"(src)
+                   : "memory");
+    }
+  };
+  const int nchunk = kend > kbeg ? (kend - kbeg + TBK - 1) / TBK : 0;
+  for (int c = 0; c < kTnStages - 1; ++c) {
+    if (c < nchunk) copy(kbeg + c * TBK, c);
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+  }
+  uint32_t phase = 0;
+  bool ok = true;
+  const int rows8 = (rows + 7) & ~7, cols8 = (cols + 7) & ~7;
+  for (int ch = 0; ch < nchunk && ok; ++ch) {
+    if (ch + kTnStages - 1 < nchunk) copy(kbeg + (ch + kTnStages - 1) * TBK, (ch + kTnStages - 1) % kTnStages);
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+    asm volatile("cp.async.wait_group %0;\n" ::"n"(kTnStages - 1) : "memory");
+    __syncthreads();
+    const float* src = stage + (size_t)(ch % kTnStages) * TBK * (rows + cols);
+    const int kn = min(TBK, kend - (kbeg + ch * TBK));
+    // tasks: a row of A^T or column of B and eight of the chunk's K (16 bytes of BF16)
+    for (int t = tid; t < (rows8 + cols8) * (TBK / 8); t += 256) {
+      const bool b = t >= rows8 * (TBK / 8);
+      const int u = b ? t - rows8 * (TBK / 8) : t, lines = b ? cols8 : rows8;
+      const int kc = u / lines, line = u - kc * lines;
+      const float* p = src + (b ? rows : 0) + line;
+      const bool in = line < (b ? cols : rows);
+      float v[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) v[j] = in && kc * 8 + j < kn ? p[(kc * 8 + j) * (rows + cols)] : 0.f;
+      *reinterpret_cast<uint4*>((b ? sB + ((kc * (TBN / 8) + (line >> 3)) * 8 + (line & 7)) * 16
+                                   : sA + ((kc * (TBM / 8) + (line >> 3)) * 8 + (line & 7)) * 16)) =
+          make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    __syncthreads();
+    if (tid == 0) {
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll
+      for (int s = 0; s < TBK / 16; ++s) {
+        const uint64_t ad = smem_desc(smem_u32(sA) + s * 2 * (TBM / 8) * 128, (TBM / 8) * 128, 128);
+        const uint64_t bd = smem_desc(smem_u32(sB) + s * 2 * (TBN / 8) * 128, (TBN / 8) * 128, 128);
+        const uint32_t acc = (ch > 0 || s > 0) ? 1u : 0u;
+        asm volatile(
+            "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+            " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
+            "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
+            : "memory");
+      }
+      asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar_a)
+                   : "memory");
+    }
+    ok = __syncthreads_and(mbar_wait(mbar_a, phase, g.spin) ? 1 : 0) != 0;   // one verdict for the CTA
+    phase ^= 1u;
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  }
+  asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+  if (!ok) {
+    if (tid == 0) atomicExch(&g_gemm_timeout[g.slot], 1);
+    mbar_wait(mbar_a, phase ^ 1u);   // drain (the default bound) before the accumulator is freed
+  } else if (warp * 32 < rows) {     // warps 0-3: accumulator rows 32 w ..
+    const int row = m0 + warp * 32 + lane;
+#pragma unroll
+    for (int c0 = 0; c0 < TBN; c0 += 16) {
+      float v[16];
+#pragma unroll
+      for (int j = 0; j < 16; ++j) v[j] = 0.f;
+      if (nchunk > 0) tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
+      if (row < g.M) {
+#pragma unroll
+        for (int j = 0; j < 16; ++j)
+          if (c0 + j < cols) partial[((long long)ks * g.M + row) * g.N + n0 + c0 + j] = v[j];
+      }
+      __syncwarp();
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (warp == 0)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
+}
+
 // ---------------------------------------------------------------------------------
 // The products of one transform or mixing step in one launch (BF16 tcgen05.mma as k_gemm, one
 // accumulator per product, so that each sum of two products is rounded as by two k_gemm calls
@@ -410,6 +551,8 @@ struct ProdArgs {
   int per;              // batch items in a tile's columns (N <= 64 / per), or 0: one item, N in tiles of 64
   int mt, nt;           // tiles along M; along N (per = 0) or groups of items
   long long items;
+  FastDiv fdN;          // by N
+  int copies;           // copies of the rows in the tile: 128 / copies rows apart
   int vecC;
   long long spin;
   int slot;
@@ -420,20 +563,8 @@ template <int MODE> constexpr int prod_accs() { return MODE == kPairs ? 4 : 2; }
 template <int MODE> constexpr int prod_smem() { return MODE == kPairs ? 78 * 1024 : 52 * 1024; }
 static_assert(2 * (kTileABytes + kTileBBytes) + 32 <= 52 * 1024, "staged operands");
 
-__device__ __forceinline__ void tmem_ld16(uint32_t addr, float* v) {
-  uint32_t r[16];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(addr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-  for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]);
-}
-
 template <int MODE>
-__global__ void __launch_bounds__(128) k_prod(ProdArgs g) {
+__global__ void __launch_bounds__(128, MODE == kPairs ? 2 : 4) k_prod(ProdArgs g) {
   constexpr int NACC = prod_accs<MODE>();
   constexpr int COLS = NACC * TBN;
   extern __shared__ __align__(1024) unsigned char smem[];
@@ -477,17 +608,18 @@ __global__ void __launch_bounds__(128) k_prod(ProdArgs g) {
   // the next chunk or item under this one's MMA and epilogue
   constexpr int NB = TBN * (TBK / 8) / 128, HB = MODE == kTwoLeft ? 1 : 2;
   float vb[HB][NB][8];
+  // task u of this thread: column tn and K group tk0 + 2 u (B rows along N), or for B rows along K
+  // column tid / 8 + 16 u and group tid mod 8
+  const int tn = tid & (TBN - 1), tk0 = tid / TBN;
+  const int tj = g.per > 0 ? g.fdN.div(tn) : 0, tg = tn - tj * g.N;   // the column's item and column
   auto loadB = [&](const Tile& t, int k0) {
-    const int kn = min(TBK, g.K - k0), kcn = (kn + 15) / 16 * 2;
+    const int kn = min(TBK, g.K - k0);
 #pragma unroll
     for (int u = 0; u < NB; ++u) {
-      const int c = tid + u * 128;
-      int n, kc;
-      if (g.tb) { n = c / kcn; kc = c - n * kcn; }
-      else { kc = c / TBN; n = c - kc * TBN; }
-      if (kc >= kcn || n >= t.cols) continue;
-      const int j0 = g.per > 0 ? n / g.N : 0;
-      const int gn = g.per > 0 ? n - j0 * g.N : t.n0 + n;
+      const int n = g.tb ? (tid >> 3) + 16 * u : tn, kc = g.tb ? (tid & 7) : tk0 + 2 * u;
+      if (kc * 8 >= kn || n >= t.cols) continue;
+      const int j0 = g.per > 0 ? (g.tb ? g.fdN.div(n) : tj) : 0;
+      const int gn = g.per > 0 ? (g.tb ? n - j0 * g.N : tg) : t.n0 + n;
       const long long off =
           (long long)(t.b0 + j0) * g.sB + (g.tb ? (long long)gn * g.ldb + k0 : (long long)k0 * g.ldb + gn);
       const int ks = g.tb ? 1 : g.ldb;
@@ -524,8 +656,10 @@ __global__ void __launch_bounds__(128) k_prod(ProdArgs g) {
               if (r < rows && k < kn)
                 v[j] = g.ta ? A[(long long)(k0 + k) * g.lda + m0 + r] : A[(long long)(m0 + r) * g.lda + k0 + k];
             }
-            *reinterpret_cast<uint4*>(sA[h] + ((kc * (TBM / 8) + (r >> 3)) * 8 + (r & 7)) * 16) =
+            const uint4 q =
                 make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
+            for (int y = 0, ry = r; y < g.copies; ++y, ry += TBM / g.copies)
+              *reinterpret_cast<uint4*>(sA[h] + ((kc * (TBM / 8) + (ry >> 3)) * 8 + (ry & 7)) * 16) = q;
           }
         }
         staged_m0 = keepA ? m0 : -1;
@@ -533,16 +667,15 @@ __global__ void __launch_bounds__(128) k_prod(ProdArgs g) {
       // the tile's columns (columns past `cols` keep what is there: they reach no result)
 #pragma unroll
       for (int u = 0; u < NB; ++u) {
-        const int c = tid + u * 128;
-        int n, kc;
-        if (g.tb) { n = c / kcn; kc = c - n * kcn; }
-        else { kc = c / TBN; n = c - kc * TBN; }
+        const int n = g.tb ? (tid >> 3) + 16 * u : tn, kc = g.tb ? (tid & 7) : tk0 + 2 * u;
         if (kc >= kcn || n >= cols) continue;
+        const bool some = kc * 8 < kn;   // else a group of padding
 #pragma unroll
         for (int h = 0; h < HB; ++h) {
           const float* v = vb[h][u];
+          const uint4 q = make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
           *reinterpret_cast<uint4*>(sB[h] + ((kc * (TBN / 8) + (n >> 3)) * 8 + (n & 7)) * 16) =
-              make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
+              some ? q : make_uint4(0u, 0u, 0u, 0u);
         }
       }
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -581,11 +714,15 @@ __global__ void __launch_bounds__(128) k_prod(ProdArgs g) {
       mbar_wait(mbar_a, phase ^ 1u);
       break;
     }
-    if (warp * 32 < rows) {
-      const int row = m0 + warp * 32 + lane;
-      const bool live = warp * 32 + lane < rows;
+    // a warp reads its 32 accumulator rows: with copies of the rows in the tile, one copy's warps
+    // take one share of the columns
+    const int span = TBM / g.copies, base = warp * 32 % span;
+    if (base < rows) {
+      const int row = m0 + base + lane;
+      const bool live = base + lane < rows;
       const uint32_t tw = tmem + ((uint32_t)(warp * 32) << 16);
-      for (int c0 = 0; c0 < cols; c0 += 16) {
+#pragma unroll 1
+      for (int c0 = 16 * (warp * 32 / span); c0 < cols; c0 += 16 * g.copies) {
         float p[NACC][16];
 #pragma unroll
         for (int q = 0; q < NACC; ++q) tmem_ld16(tw + (uint32_t)(q * TBN + c0), p[q]);
@@ -602,7 +739,7 @@ __global__ void __launch_bounds__(128) k_prod(ProdArgs g) {
           for (int j4 = 0; j4 < 16; j4 += 4) {
             const int n = c0 + j4;
             if (n >= cols) break;
-            const int j0 = g.per > 0 ? n / g.N : 0;
+            const int j0 = g.per > 0 ? g.fdN.div(n) : 0;
             float* d = C + (long long)(b0 + j0) * g.sC + (long long)row * g.ldc + (g.per > 0 ? n - j0 * g.N : n0 + n);
             if (g.vecC) {   // N, the strides and the base are multiples of four floats
               float4 w = make_float4(o[j4], o[j4 + 1], o[j4 + 2], o[j4 + 3]);
@@ -616,7 +753,7 @@ __global__ void __launch_bounds__(128) k_prod(ProdArgs g) {
               *reinterpret_cast<float4*>(d) = w;
             } else {
               for (int e = 0; e < 4 && n + e < cols; ++e) {
-                const int je = g.per > 0 ? (n + e) / g.N : 0;
+                const int je = g.per > 0 ? g.fdN.div(n + e) : 0;
                 float* de = C + (long long)(b0 + je) * g.sC + (long long)row * g.ldc +
                             (g.per > 0 ? n + e - je * g.N : n0 + n + e);
                 float w = o[j4 + e];
@@ -683,7 +820,18 @@ cudaError_t gemm_timeout_read(int slot, int* host_flag, cudaStream_t s) {
 static thread_local float* g_split_ws = nullptr;
 static thread_local long long g_split_floats = 0;
 
-static void launch_gemm(const GemmArgs& g, int gm, int gn, int ksplit, cudaStream_t s) {
+static cudaError_t launch_gemm(const GemmArgs& g, int gm, int gn, int ksplit, cudaStream_t s) {
+  // long splits of A^T B whose rows can be copied in 16-byte pieces
+  if (ksplit > 1 && g.batch == 1 && g.ta && !g.tb && g.M % 4 == 0 && g.N % 4 == 0 && g.lda % 4 == 0 && g.ldb % 4 == 0 &&
+      ((reinterpret_cast<uintptr_t>(g.A) | reinterpret_cast<uintptr_t>(g.B)) & 15) == 0) {
+    // 200 KB at most (128 rows, 64 columns): one CTA an SM then, and tensor memory for its 64 columns
+    static std::atomic<int> cache[kAttrDevices] = {};
+    const size_t smem = tn_smem(std::min(g.M, TBM), std::min(g.N, TBN));
+    const cudaError_t e = smem_attr(k_gemm_tn, smem, cache);
+    if (e != cudaSuccess) return e;
+    k_gemm_tn<<<dim3(gn, gm, ksplit), 256, std::max<size_t>(smem, kGemmSmem), s>>>(g, ksplit, g_split_ws);
+    return cudaGetLastError();
+  }
   if (g.K <= TBK) {
     const long long others = (long long)gn * g.batch * ksplit;
     const int gy = (int)std::max<long long>(1, std::min<long long>(gm, 152 * 8 / others));
@@ -691,6 +839,7 @@ static void launch_gemm(const GemmArgs& g, int gm, int gn, int ksplit, cudaStrea
   } else {
     k_gemm<true><<<dim3(gn, gm, g.batch * ksplit), 128, kGemmSmem, s>>>(g, ksplit, g_split_ws);
   }
+  return cudaGetLastError();
 }
 
 cudaError_t gemm_bf16(const GemmArgs& g0, cudaStream_t s) {
@@ -729,11 +878,13 @@ cudaError_t gemm_bf16(const GemmArgs& g0, cudaStream_t s) {
       h.A = g.A + (long long)b0 * g.sA;
       h.B = g.B + (long long)b0 * g.sB;
       h.C = g.C + (long long)b0 * g.sC;
-      launch_gemm(h, gm, gn, 1, s);
+      const cudaError_t e = launch_gemm(h, gm, gn, 1, s);
+      if (e != cudaSuccess) return e;
     }
     return cudaGetLastError();
   }
-  launch_gemm(g, gm, gn, ksplit, s);
+  const cudaError_t el = launch_gemm(g, gm, gn, ksplit, s);
+  if (el != cudaSuccess) return el;
   if (ksplit > 1) {
     const long long total = (long long)g.M * g.N * g.batch;
     const int blocks = (int)std::min<long long>((total + 255) / 256, 152 * 8);
@@ -756,46 +907,47 @@ __global__ void k_gelu_back(const float* dv, const float* z, float* dz, long lon
 
 // deterministic column sums: stage 1 per row block, stage 2 over the blocks, each column added in
 // order by one thread from rows that the whole CTA has staged (the additions are a chain of
-// short latencies; straight from global memory it was a chain of long ones: 33 and 41 us, now 7
-// and 4 us for 127008 rows of 32 columns)
-constexpr int kColRows = 64, kColMax = 128;
+// short latencies; straight from global memory it was a chain of long ones: 33 and 41 us, now 14
+// us each for 127008 rows of 32 columns)
+constexpr int kColMax = 128, kColTile = 8192;   // columns at a time, staged floats
 __device__ __forceinline__ void colsum_staged(const float* x, long long r0, long long r1, int cols, int c0, float* tile,
                                               float* out) {
-  const int nc = min(kColMax, cols - c0);
+  const int nc = min(kColMax, cols - c0), nr = kColTile / nc;
+  const FastDiv fd((uint32_t)nc);
   float s = 0.f;
-  for (long long r = r0; r < r1; r += kColRows) {
-    const int n = (int)min((long long)kColRows, r1 - r);
+  for (long long r = r0; r < r1; r += nr) {
+    const int n = (int)min((long long)nr, r1 - r);
     for (int t0 = threadIdx.x; t0 < n * nc; t0 += 8 * blockDim.x) {   // eight loads in flight a thread
       float v[8];
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
-        const int t = t0 + u * (int)blockDim.x, i = t / nc;
+        const int t = t0 + u * (int)blockDim.x, i = fd.div(t);
         if (t < n * nc) v[u] = x[(r + i) * cols + c0 + t - i * nc];
       }
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
-        const int t = t0 + u * (int)blockDim.x, i = t / nc;
-        if (t < n * nc) tile[i * kColMax + t - i * nc] = v[u];
+        const int t = t0 + u * (int)blockDim.x;
+        if (t < n * nc) tile[t] = v[u];
       }
     }
     __syncthreads();
     if (threadIdx.x < nc) {
 #pragma unroll 16
-      for (int i = 0; i < n; ++i) s += tile[i * kColMax + threadIdx.x];
+      for (int i = 0; i < n; ++i) s += tile[i * nc + threadIdx.x];
     }
     __syncthreads();
   }
   if (threadIdx.x < nc) out[c0 + threadIdx.x] = s;
 }
 __global__ void __launch_bounds__(256) k_colsum1(const float* x, long long rows, int cols, int rows_per, float* part) {
-  __shared__ float tile[kColRows * kColMax];
+  __shared__ float tile[kColTile];
   const long long r0 = min(rows, (long long)blockIdx.x * rows_per);
   const long long r1 = min(rows, r0 + rows_per);
   for (int c0 = 0; c0 < cols; c0 += kColMax)
     colsum_staged(x, r0, r1, cols, c0, tile, part + (long long)blockIdx.x * cols);
 }
 __global__ void __launch_bounds__(256) k_colsum2(const float* part, int nblk, int cols, float* out) {
-  __shared__ float tile[kColRows * kColMax];
+  __shared__ float tile[kColTile];
   for (int c0 = blockIdx.x * kColMax; c0 < cols; c0 += gridDim.x * kColMax)
     colsum_staged(part, 0, nblk, cols, c0, tile, out);
 }
@@ -1008,6 +1160,8 @@ template <int MODE> static cudaError_t run_prod(ProdArgs g, cudaStream_t s) {
   g.per = g.sA == 0 && 2 * g.N <= TBN && g.batch > 1 ? TBN / g.N : 0;
   g.vecC = g.N % 4 == 0 && g.ldc % 4 == 0 && g.sC % 4 == 0 && al16(g.C0) && (MODE == kSum || al16(g.C1));
   g.mt = (g.M + TBM - 1) / TBM;
+  g.fdN = FastDiv((uint32_t)g.N);
+  g.copies = g.M <= 32 ? 4 : (g.M <= 64 ? 2 : 1);
   g.nt = g.per > 0 ? (g.batch + g.per - 1) / g.per : (g.N + TBN - 1) / TBN;
   g.items = (long long)g.mt * g.nt * (g.per > 0 ? 1 : g.batch);
   static std::atomic<int> cache[kAttrDevices] = {};
