@@ -172,6 +172,7 @@ struct Geometry {
   double A0[3][3];
   std::vector<hom_inclusion> incl;
   FftPlan plan[3];
+  FftPlan planff[3];   // of the float-float passes (no composite radices)
   // pixel image of an isotropic conductivity ([P2][P1] or [P3][P2][P1], x fastest), or empty
   std::vector<double> bitmap;
   int P[3] = {1, 1, 1};
@@ -364,7 +365,10 @@ hom_status build_geometry(hom_ctx* ctx, const hom_problem* P, Geometry& g, bool 
   g.planes = (long long)g.M[1] * g.M[2];
   g.grid = g.planes * g.M[0];
   g.spec = g.planes * g.Nxs;
-  for (int a = 0; a < 3; ++a) make_plan(g.M[a], g.plan[a]);
+  for (int a = 0; a < 3; ++a) {
+    make_plan(g.M[a], g.plan[a]);
+    make_plan(g.M[a], g.planff[a], false);
+  }
   return HOM_OK;
 }
 
@@ -845,6 +849,7 @@ struct Runner {
                     const void* r_aux, const void* p_aux, int prologue, const void* bsub = nullptr) {
     constexpr bool ff = is_ff<T>::value;   // float-float: in and out FP64, passes in FP32 pairs
     auto W = [&](int a) -> const void* { return base + (ff ? L.twff[a] : sizeof(T) == 8 ? L.tw64[a] : L.tw32[a]); };
+    auto plan = [&](int a) -> const FftPlan& { return ff ? g.planff[a] : g.plan[a]; };
     const int C = g.d;
     const int Mx = g.M[0], My = g.M[1], Mz = g.M[2];
     const int Ny = g.N[1], Nz = g.N[2], Nh = g.Nh;
@@ -859,7 +864,7 @@ struct Runner {
       z.nslab = R * C; z.X = Ny * Nh; z.XC = pencil_xc<T>(Mz, z.X, 1, z.nslab);
       z.Pin = Nz; z.Pout = Mz; z.Nlog = Nz; z.dir = +1;
       z.slabs_per_rhs = C; z.slabs_per_comp = 1; z.C = C; z.prologue = prologue;
-      z.W = W(2); z.plan = g.plan[2]; z.cg = cg; z.in64 = ff;
+      z.W = W(2); z.plan = plan(2); z.cg = cg; z.in64 = ff;
       if (sizeof(T) == 4 && (ctx->zpipe_mask & 2))
         z.pgrid = zpipe_pad_grid(Mz, z.Pin, z.Pout, z.Nlog, z.dir, z.X, z.nslab, ctx->sms);
       if (z.XC < 1) return fail(ctx, HOM_ERR_INVALID_ARG, "grid too large for the shared-memory FFT");
@@ -893,7 +898,7 @@ struct Runner {
       y.Pin = Ny; y.Pout = My; y.Nlog = Ny; y.dir = +1;
       y.slabs_per_rhs = C * Mz; y.slabs_per_comp = Mz; y.C = C;
       y.prologue = g.d == 3 ? 0 : prologue;
-      y.W = W(1); y.plan = g.plan[1]; y.cg = cg; y.in64 = ff && g.d == 2;
+      y.W = W(1); y.plan = plan(1); y.cg = cg; y.in64 = ff && g.d == 2;
       if (y.XC < 1) return fail(ctx, HOM_ERR_INVALID_ARG, "grid too large for the shared-memory FFT");
       KL(launch_pencil<T>(y, st));
     }
@@ -905,7 +910,7 @@ struct Runner {
                                : xpass_yb<T>(Mx, C, (int)g.planes, R);
       x.Nin = Nh; x.Nout = Nh; x.M = Mx; x.R = R; x.C = C; x.ncomp = g.ncomp; x.d = g.d;
       x.comp_stride = g.planes * Nh; x.scale = 1.0 / (double)g.grid;
-      x.W = W(0); x.plan = g.plan[0]; x.cg = cg; x.partial = nullptr;
+      x.W = W(0); x.plan = plan(0); x.cg = cg; x.partial = nullptr;
       if (x.YB < 1) return fail(ctx, HOM_ERR_INVALID_ARG, "grid too large for the shared-memory FFT");
       KL(launch_xpass<T>(x, R, st));
     }
@@ -917,7 +922,7 @@ struct Runner {
       y.nslab = R * C * Mz; y.X = Nh; y.XC = ctx->ypass_xc > 0 ? chunk(pencil_xc<T>(My, Nh, 1), ctx->ypass_xc) : pencil_xc<T>(My, Nh, 1, y.nslab);
       y.Pin = My; y.Pout = Ny; y.Nlog = Ny; y.dir = -1;
       y.slabs_per_rhs = C * Mz; y.slabs_per_comp = Mz; y.C = C; y.prologue = 0;
-      y.W = W(1); y.plan = g.plan[1]; y.cg = cg;
+      y.W = W(1); y.plan = plan(1); y.cg = cg;
       KL(launch_pencil<T>(y, st));
       fin = T1;
     }
@@ -933,7 +938,7 @@ struct Runner {
       f.nrhs = R; f.C = C; f.XC = pencil_xc<T>(Mlast, f.X, C, R); f.M = Mlast; f.Nlog = Nlast;
       f.project = project; f.d = g.d; f.Ny = Ny; f.Nh = Nh;
       for (int k = 0; k < 3; ++k) f.invY[k] = g.invY[k];
-      f.W = W(g.d == 3 ? 2 : 1); f.plan = g.plan[g.d == 3 ? 2 : 1];
+      f.W = W(g.d == 3 ? 2 : 1); f.plan = plan(g.d == 3 ? 2 : 1);
       f.cg = cg; f.partial_ld = L.maxblk; f.bsub = bsub;
       f.partial = ((cg && p_aux) || bsub) ? at<double>(L.partial) : nullptr;
       if (sizeof(T) == 4 && !bsub) {
@@ -1669,7 +1674,10 @@ Geometry gani_geometry(const Geometry& g) {
   n.planes = (long long)n.M[1] * n.M[2];
   n.grid = n.planes * n.M[0];
   n.spec = n.planes * n.Nxs;
-  for (int a = 0; a < 3; ++a) make_plan(n.M[a], n.plan[a]);
+  for (int a = 0; a < 3; ++a) {
+    make_plan(n.M[a], n.plan[a]);
+    make_plan(n.M[a], n.planff[a], false);
+  }
   return n;
 }
 

@@ -159,8 +159,8 @@ __host__ __device__ inline void plan_divisions(FftPlan& p) {
 // Radices of a transform of length M: primes above 13 first (their first inverse stage skips
 // the zero padding's terms and needs no twiddles), then with `big` the composite register
 // radices 15 and 9 (fewer passes through shared memory), then 13, 11, 7, 5, 3 and, for image
-// lengths and even grids (the double grid is odd), 8, 4, 2. The batched kernel takes radices
-// 5, 3, 7, 11, 13 in this order (big = false, see fft_pencils_small).
+// lengths and even grids (the double grid is odd), 8, 4, 2. The batched kernel and float-float
+// passes take radices 5, 3, 7, 11, 13 in this order (big = false, see fft_pencils_small and cfft).
 inline void make_plan(int M, FftPlan& p, bool big = true) {
   p.M = M;
   p.nrad = 0;
@@ -785,9 +785,21 @@ __device__ __forceinline__ cpx<T>* fft_plan_run(cpx<T>* a, cpx<T>* b, int G, int
       HOMB_STAGE(7)
       HOMB_STAGE(11)
       HOMB_STAGE(13)
-      HOMB_STAGE(9)
-      HOMB_STAGE(15)
       default:
+        if constexpr (!is_ff<T>::value) {   // float-float plans hold no composite radix
+          if (R == 9) {
+            if (DIR > 0 && zi) stage_radix<T, 9, DIR, (DIR > 0), false>(src, dst, G, ld, M, Ns, dnb, dns, W);
+            else if (DIR < 0 && zo) stage_radix<T, 9, DIR, false, (DIR < 0)>(src, dst, G, ld, M, Ns, dnb, dns, W);
+            else stage_radix<T, 9, DIR, false, false>(src, dst, G, ld, M, Ns, dnb, dns, W);
+            break;
+          }
+          if (R == 15) {
+            if (DIR > 0 && zi) stage_radix<T, 15, DIR, (DIR > 0), false>(src, dst, G, ld, M, Ns, dnb, dns, W);
+            else if (DIR < 0 && zo) stage_radix<T, 15, DIR, false, (DIR < 0)>(src, dst, G, ld, M, Ns, dnb, dns, W);
+            else stage_radix<T, 15, DIR, false, false>(src, dst, G, ld, M, Ns, dnb, dns, W);
+            break;
+          }
+        }
         {
           int qn = (R - 1) / 2, sn = (R - 1) / 2;
           if (DIR > 0 && (band.prune & 1) && i == 0)   // pairs with a position <= half or >= M - top
@@ -1044,14 +1056,16 @@ __device__ __forceinline__ cpx<T>* cfft_from(cpx<T>* a, cpx<T>* b, int G, const 
 }
 
 // G contiguous pencils of compile-time length M (stride M), ping-pong between a and b.
-// FP32 and float-float use the composite register radices (fewer shared-memory passes, and
-// no twiddle products inside a prime-factor radix 15); FP64 keeps
-// radices 3 and 5, which need the fewest FP64 operations, except at M = 225 = 15 * 15, where
-// the radix-15 stages with the zero band pruned (bits 4 and 8) need fewer.
+// FP32 uses the composite register radices (fewer shared-memory passes, and no twiddle products
+// inside a prime-factor radix 15); FP64 keeps radices 3 and 5, which need the fewest FP64
+// operations, and so does float-float, whose composite radices leave a chunk of pencils too few
+// butterflies for a CTA's threads (radix 25 at length 125: 55 of 256) and take 255 registers a
+// thread (the float-float operator at N = 63: 1.68 ms; 0.69 ms with radices 5 and two CTAs an SM), except at M = 225 = 15 * 15, where the
+// radix-15 stages with the zero band pruned (bits 4 and 8) need fewer operations.
 constexpr int kBandM64 = 225;
 template <typename T, int M>
 __device__ __forceinline__ cpx<T>* cfft(cpx<T>* a, cpx<T>* b, int G, const cpx<T>* W, int dir, int prune = 0) {
-  return cfft_from<T, M, 0, (sizeof(T) == 4 || is_ff<T>::value || M == kBandM64)>(a, b, G, W, dir, prune);
+  return cfft_from<T, M, 0, (sizeof(T) == 4 || M == kBandM64)>(a, b, G, W, dir, prune);
 }
 
 // Prune bits valid for a length-M transform whose spectrum is nonzero (inverse) or needed

@@ -19,6 +19,8 @@
 namespace homb {
 
 constexpr int kPassThreads = 256;
+// float-float: at most 128 registers a thread, two CTAs an SM (its dependent chains need the warps)
+template <typename T> constexpr int pass_min_ctas() { return is_ff<T>::value ? 2 : 0; }   // 0: none asked
 #ifndef HOMB_PASS_SMEM_KB
 #define HOMB_PASS_SMEM_KB 48
 #endif
@@ -109,7 +111,7 @@ __device__ __forceinline__ void fft_warp_all(cpx<T>* A, int G, const cpx<T>* Wt,
 // pencil pass along y or z (one component slab per CTA, XC contiguous positions)
 // ---------------------------------------------------------------------------------
 template <typename T, int MT>
-__global__ void __launch_bounds__(kPassThreads) k_pencil(PencilArgs a) {
+__global__ void __launch_bounds__(kPassThreads, pass_min_ctas<T>()) k_pencil(PencilArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int M = MT > 0 ? MT : a.plan.M;
   cpx<T>* Ws = reinterpret_cast<cpx<T>*>(smem);
@@ -207,7 +209,7 @@ __global__ void __launch_bounds__(kPassThreads) k_pencil(PencilArgs a) {
 // final forward pass + truncation + projection (+ CG partial p.q or FP64 residual)
 // ---------------------------------------------------------------------------------
 template <typename T, int MT>
-__global__ void __launch_bounds__(kPassThreads) k_final(FinalArgs a) {
+__global__ void __launch_bounds__(kPassThreads, pass_min_ctas<T>()) k_final(FinalArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int M = MT > 0 ? MT : a.M;
   const int C = a.C;
@@ -421,7 +423,9 @@ __device__ __forceinline__ void apply_coef(const T* coef, long long gi, long lon
                                            int d, const T* u, T* v, T scale) {
   if (ncomp == 1) {
     const T a = coef[gi] * scale;
-    for (int c = 0; c < d; ++c) v[c] = a * u[c];
+#pragma unroll
+    for (int c = 0; c < 3; ++c)   // a constant trip count keeps u and v in registers
+      if (c < d) v[c] = a * u[c];
   } else if (d == 2) {
     const T a11 = coef[gi] * scale, a22 = coef[gi + cstride] * scale, a12 = coef[gi + 2 * cstride] * scale;
     v[0] = fma(a11, u[0], a12 * u[1]);
@@ -520,7 +524,7 @@ __device__ __forceinline__ void xpass_warp(const XArgs& a, cpx<T>* Ws, cpx<T>* A
 }
 
 template <typename T, int MT>
-__global__ void __launch_bounds__(kPassThreads) k_xpass(XArgs a) {
+__global__ void __launch_bounds__(kPassThreads, pass_min_ctas<T>()) k_xpass(XArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int M = MT > 0 ? MT : a.M;
   const int p0 = blockIdx.x * a.YB;
