@@ -911,6 +911,7 @@ struct Runner {
       x.Nin = Nh; x.Nout = Nh; x.M = Mx; x.R = R; x.C = C; x.ncomp = g.ncomp; x.d = g.d;
       x.comp_stride = g.planes * Nh; x.scale = 1.0 / (double)g.grid;
       x.W = W(0); x.plan = plan(0); x.cg = cg; x.partial = nullptr;
+      x.pair = ctx->xpass_yb > 0 ? 0 : 1;   // a caller's planes per CTA keep the single-pair pass
       if (x.YB < 1) return fail(ctx, HOM_ERR_INVALID_ARG, "grid too large for the shared-memory FFT");
       KL(launch_xpass<T>(x, R, st));
     }

@@ -14,6 +14,7 @@ template <> struct cplx_t<float> { using type = float2; };
 namespace homb {
 template <> struct cplx_t<ffloat> { using type = ffloat2; };
 template <typename T> using cpx = typename cplx_t<T>::type;
+template <typename T> struct is_fpair { static constexpr bool value = false; };   // fpair.cuh
 
 template <typename T> __device__ __forceinline__ cpx<T> mk(T x, T y) { cpx<T> r; r.x = x; r.y = y; return r; }
 template <typename T> __device__ __forceinline__ cpx<T> add(cpx<T> a, cpx<T> b) { return mk<T>(a.x + b.x, a.y + b.y); }
@@ -1065,7 +1066,7 @@ __device__ __forceinline__ cpx<T>* cfft_from(cpx<T>* a, cpx<T>* b, int G, const 
 constexpr int kBandM64 = 225;
 template <typename T, int M>
 __device__ __forceinline__ cpx<T>* cfft(cpx<T>* a, cpx<T>* b, int G, const cpx<T>* W, int dir, int prune = 0) {
-  return cfft_from<T, M, 0, (sizeof(T) == 4 || M == kBandM64)>(a, b, G, W, dir, prune);
+  return cfft_from<T, M, 0, (sizeof(T) == 4 || is_fpair<T>::value || M == kBandM64)>(a, b, G, W, dir, prune);
 }
 
 // Prune bits valid for a length-M transform whose spectrum is nonzero (inverse) or needed

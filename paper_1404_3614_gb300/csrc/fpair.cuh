@@ -7,6 +7,8 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include "common.cuh"
+
 namespace homb {
 // in a namespace of its own, as ffloat: found by argument-dependent lookup
 namespace fpa {
@@ -37,5 +39,7 @@ __device__ __forceinline__ fpair fma(fpair a, fpair b, fpair c) { return fp(__ff
 
 using fpa::fpair;
 using fpa::fpair2;
+template <> struct cplx_t<fpair> { using type = fpair2; };
+template <> struct is_fpair<fpair> { static constexpr bool value = true; };
 
 }  // namespace homb

@@ -73,6 +73,7 @@ struct XArgs {
   FftPlan plan;
   CgScalars* cg;
   double* partial;        // mode 1: [gridDim.x][R*R]
+  int pair;               // FP32 mode 0: packed double pencils, the pass's own planes per CTA (YB unused)
   FastDiv fd_Nin, fd_Nout, fd_rpp;   // set by the launcher
 };
 

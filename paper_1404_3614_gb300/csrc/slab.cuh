@@ -23,8 +23,6 @@
 
 namespace homb {
 
-template <> struct cplx_t<fpair> { using type = fpair2; };
-
 constexpr int kSlabMaxThreads = 480;   // 15 warps: up to 136 registers a thread
 
 // Layout of the slab in shared memory: columns kx = l + R m and l + R (m + 1), m even, side by side
