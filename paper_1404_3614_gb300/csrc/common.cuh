@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <initializer_list>
+
 namespace homb {
 
 template <typename T> struct cplx_t;
@@ -220,8 +222,8 @@ template <typename T> __device__ __forceinline__ void dft5(cpx<T>* v, int dir) {
   v[3] = sub<T>(m2, in2);
 }
 
-// Compile-time cos / sin of 2 pi p / q from their Taylor series (argument reduced to
-// [-pi, pi]); used only for the twiddle constants inside the register DFTs.
+// Compile-time cos / sin from their Taylor series (arguments up to pi / 4); used only for the
+// twiddle constants inside the register DFTs.
 __host__ __device__ constexpr double ct_sin_red(double x) {
   double term = x, sum = x;
   for (int n = 1; n < 30; ++n) {
@@ -238,15 +240,38 @@ __host__ __device__ constexpr double ct_cos_red(double x) {
   }
   return sum;
 }
-// angle 2 pi p / q reduced to (-pi, pi]
-__host__ __device__ constexpr double ct_angle(int p, int q) {
+// cos and sin of 2 pi p / q, reduced in integers to an angle 2 pi n / m of the first octant: there the
+// series has no cancellation (from the whole half circle it left 1e-15, seen in FP64 transforms
+// of lengths with radices 7 to 13)
+struct CtSinCos {
+  double c, s;
+};
+__host__ __device__ constexpr CtSinCos ct_octant(int n, int m) {   // 0 <= 8 n <= m
+  const double x = 6.283185307179586476925286766559 * (double)n / (double)m;
+  return CtSinCos{ct_cos_red(x), ct_sin_red(x)};
+}
+__host__ __device__ constexpr CtSinCos ct_quadrant(int n, int m) {   // 0 <= 4 n <= m
+  if (8 * n <= m) return ct_octant(n, m);
+  const CtSinCos r = ct_octant(m - 4 * n, 4 * m);   // pi / 2 less the angle
+  return CtSinCos{r.s, r.c};
+}
+__host__ __device__ constexpr CtSinCos ct_sincos(int p, int q) {
   int r = p % q;
   if (r < 0) r += q;
-  if (2 * r > q) r -= q;
-  return 6.283185307179586476925286766559 * (double)r / (double)q;
+  const bool lower = 2 * r > q;   // sin < 0
+  if (lower) r = q - r;
+  CtSinCos v{1.0, 0.0};
+  if (4 * r <= q) {
+    v = ct_quadrant(r, q);
+  } else {
+    v = ct_quadrant(q - 2 * r, 2 * q);   // pi less the angle
+    v.c = -v.c;
+  }
+  if (lower) v.s = -v.s;
+  return v;
 }
-__host__ __device__ constexpr double ct_cos2pi(int p, int q) { return ct_cos_red(ct_angle(p, q)); }
-__host__ __device__ constexpr double ct_sin2pi(int p, int q) { return ct_sin_red(ct_angle(p, q)); }
+__host__ __device__ constexpr double ct_cos2pi(int p, int q) { return ct_sincos(p, q).c; }
+__host__ __device__ constexpr double ct_sin2pi(int p, int q) { return ct_sincos(p, q).s; }
 
 __host__ __device__ constexpr int ct_first_factor(int R) {
   return R % 3 == 0 ? 3 : (R % 5 == 0 ? 5 : R);

@@ -689,7 +689,7 @@ __global__ void __launch_bounds__(kPassThreads, pass_min_ctas<T>()) k_xpass(XArg
   const long long cstride = (long long)a.planes * M;
   if (a.mode == 0) {
     const int C = a.C;
-    const T scale = T(a.scale);
+    const T scale = T(0.5 * a.scale);   // with the 1/2 of the split into rows below
     for (int t = threadIdx.x; t < YB * M; t += blockDim.x) {
       const int yy = t / M;
       const int x = t - yy * M;
@@ -723,8 +723,8 @@ __global__ void __launch_bounds__(kPassThreads, pass_min_ctas<T>()) k_xpass(XArg
       const cpx<T> zk = r2[pp * M + k];
       const cpx<T> zm = r2[pp * M + (k == 0 ? 0 : M - k)];
       cpx<T> X;
-      if ((row & 1) == 0) X = mk<T>(T(0.5) * (zk.x + zm.x), T(0.5) * (zk.y - zm.y));
-      else X = mk<T>(T(0.5) * (zk.y + zm.y), T(-0.5) * (zk.x - zm.x));
+      if ((row & 1) == 0) X = mk<T>(zk.x + zm.x, zk.y - zm.y);
+      else X = mk<T>(zk.y + zm.y, zm.x - zk.x);
       out[row_off(row) + k] = X;
     }
   } else if (a.mode == 1) {

@@ -442,8 +442,7 @@ __global__ void __launch_bounds__(kSlabMaxThreads) k_slab(SlabArgs a) {
       for (int k = 0; k < R; ++k) v[k].y = v[k].y * ce[k];
       // forward transform: lane l holds x[l + R n2] with n2 = k1; the kept frequencies only
       dft_reg<F, R>(v, -1);
-      slab_twiddle<R>(v, Ws, l, false);
-      v[0] = scl<F>(v[0], F(fs));
+      slab_twiddle<R>(v, Wt, l, false);
       slab_exchange<R>(v, Sw, l, act);
       if constexpr (ZB) dft_reg_zout<F, R>(v, -1);
       else dft_reg<F, R>(v, -1);
@@ -501,7 +500,8 @@ __global__ void __launch_bounds__(kSlabMaxThreads) k_slab(SlabArgs a) {
 #pragma unroll
       for (int n = 0; n < R; ++n) v[n] = p[l + R * n];
       dft_reg<F, R>(v, -1);
-      slab_twiddle<R>(v, Wt, l, false);
+      slab_twiddle<R>(v, Ws, l, false);
+      v[0] = scl<F>(v[0], F(fs));
       slab_exchange<R>(v, p, l, on);
       if constexpr (ZB) dft_reg_zout<F, R>(v, -1);
       else dft_reg<F, R>(v, -1);
