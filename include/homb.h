@@ -488,15 +488,17 @@ hom_status hom_matvec_noalloc(hom_ctx* ctx, const hom_problem* prob, int32_t sid
                               const void* d_coef, const void* d_in, void* d_out, void* stream);
 
 /* Tuning: pencils per CTA of the operator's y passes and planes per CTA of its row pass
- * (0: automatic, the shared-memory budget's maximum; larger requests are capped to it). */
+ * (0: automatic, the shared-memory budget's maximum, less on grids so small that it would leave
+ * multiprocessors idle; larger requests are capped to the maximum). A row-pass request also runs the
+ * FP32 operator's rows as pairs, not four at a time; results agree to rounding. */
 hom_status hom_set_pass_chunks(hom_ctx* ctx, int32_t ypass_pencils, int32_t xpass_planes);
 /* The 3D operator with an isotropic coefficient and equal x and y transform lengths
  * M = R * R (R in 3, 5, 9, 15) fuses the inverse y transforms, the x row pass and the
  * forward y transforms into one pass over (rhs, component, z) slabs held in shared memory,
  * by persistent CTAs that stage each slab's input with a bulk asynchronous copy issued
  * while the previous slab is still being transformed (enable = 1, the default: warps per
- * CTA chosen from the slab's shared memory; 4..20 in steps of 4 asks for that many warps
- * where they fit). enable = 0 runs them as three separate passes; the results agree to
+ * CTA chosen from the slab's shape; 4..20 in steps of 4 asks for that many warps where they
+ * fit, at most 15, and leaves the automatic choice where they do not). enable = 0 runs them as three separate passes; the results agree to
  * rounding. A staged copy that does not complete within a bounded wait makes hom_bounds
  * return HOM_ERR_TIMEOUT. Applies to later calls on this context. */
 hom_status hom_set_slab_pass(hom_ctx* ctx, int32_t enable);

@@ -1086,8 +1086,9 @@ __device__ __forceinline__ cpx<T>* cfft_from(cpx<T>* a, cpx<T>* b, int G, const 
 // inside a prime-factor radix 15); FP64 keeps radices 3 and 5, which need the fewest FP64
 // operations, and so does float-float, whose composite radices leave a chunk of pencils too few
 // butterflies for a CTA's threads (radix 25 at length 125: 55 of 256) and take 255 registers a
-// thread (the float-float operator at N = 63: 1.68 ms; 0.69 ms with radices 5 and two CTAs an SM), except at M = 225 = 15 * 15, where the
-// radix-15 stages with the zero band pruned (bits 4 and 8) need fewer operations.
+// thread (the float-float operator at N = 63: 1.68 ms; 0.69 ms with radices 5 and two CTAs an SM),
+// except at M = 225 = 15 * 15, where the radix-15 stages with the zero band pruned (bits 4 and 8)
+// need fewer operations.
 constexpr int kBandM64 = 225;
 template <typename T, int M>
 __device__ __forceinline__ cpx<T>* cfft(cpx<T>* a, cpx<T>* b, int G, const cpx<T>* W, int dir, int prune = 0) {

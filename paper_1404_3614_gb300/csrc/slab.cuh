@@ -596,7 +596,8 @@ template <typename T> cudaError_t launch_slab(const SlabArgs& a, cudaStream_t s)
     int warps = slab_warps<T>(a.M, a.Ny, a.Nh);
     if (warps && a.warps > 0) {   // a caller's choice, where it fits
       const int r = a.M == 225 ? 15 : (a.M == 81 ? 9 : (a.M == 25 ? 5 : 3));
-      if (a.warps * 32 <= kSlabMaxThreads && slab_smem_bytes(r, slab_band_free(a.M, a.Ny, a.Nh), a.Ny, a.Nh, a.warps) <= 220 * 1024)
+      const bool zb = slab_band_free(a.M, a.Ny, a.Nh);
+      if (a.warps * 32 <= kSlabMaxThreads && slab_smem_bytes(r, zb, a.Ny, a.Nh, a.warps) <= 220 * 1024)
         warps = a.warps;
     }
     switch (warps ? a.M : 0) {
