@@ -59,11 +59,11 @@ def measured_peaks():
         return {"hbm_gbs": FALLBACK_HBM_GBS, "source": "of fallback (recipe: 6.8 TB/s)"}
 
 
-# DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of one k_slab<float, 15> launch on
+# DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of one k_slab<15> launch on
 # the 16-ball cell (9 fields, 3 right-hand sides), from one ncu capture of the build whose
 # kernel sources (the kernel's file, the device helpers it calls and its argument struct) hash
 # to `sha256_16`; reported only while they still do.
-SLAB_TRAFFIC = {"sha256_16": "54945fc3d6ddd343", "bytes": 149977344 + 48060672,
+SLAB_TRAFFIC = {"sha256_16": "9e64942ae403aa11", "bytes": 149978368 + 50548480,
                 "sources": ("common.cuh", "kernels.cuh:SlabArgs", "slab.cuh"),
                 "capture": "profiles/slab_f32_spheres3d_N113.md"}
 
@@ -659,7 +659,7 @@ def extras(args, hb, solver, problem, prec, dev, stream, flush, peaks, ms_step):
         ms_l = f32["profiled_launch_ms"]
         achieved = byt / (ms_l * 1e-3) / 1e9
         res["roofline"] = {
-            "bound": "hbm", "kernel": "k_slab<float,15>", "achieved": achieved, "peak": peaks["hbm_gbs"],
+            "bound": "hbm", "kernel": "k_slab<15,true>", "achieved": achieved, "peak": peaks["hbm_gbs"],
             "unit": "GB/s", "frac": achieved / peaks["hbm_gbs"], "traffic": slab_traffic(),
             "algorithmic_bytes_per_launch": byt, "avg_launch_ms": ms_l, "launches_timed": f32["profiled_launches"],
             "peak_note": peaks["source"],
