@@ -48,6 +48,7 @@ struct GemmArgs {
   const float* bias = nullptr;   // per column, added to C; then V (leading dimension ldc), if given,
   float* V = nullptr;            // takes its activation (act: GELU, else the sum itself)
   int act = 0;
+  int drop = 0;           // with V: C is read (beta) but not written, nothing needs the sum itself
 };
 cudaError_t gemm_bf16(const GemmArgs& g, cudaStream_t s);
 // Number of per-context GEMM timeout flags; context k uses flag k mod kGemmFlagSlots.
