@@ -163,7 +163,9 @@ __host__ __device__ inline void plan_divisions(FftPlan& p) {
 // the zero padding's terms and needs no twiddles), then with `big` the composite register
 // radices 15 and 9 (fewer passes through shared memory), then 13, 11, 7, 5, 3 and, for image
 // lengths and even grids (the double grid is odd), 8, 4, 2. The batched kernel and float-float
-// passes take radices 5, 3, 7, 11, 13 in this order (big = false, see fft_pencils_small and cfft).
+// passes take radices 5, 3, 7, 11, 13 in this order (big = false, see fft_pencils_small and cfft),
+// then 8, 4, 2 as well: float-float transforms of an even grid's own length (GaNi) have them, the
+// batch has odd grids alone. Without a factor 2 left, every further radix is an odd prime.
 inline void make_plan(int M, FftPlan& p, bool big = true) {
   p.M = M;
   p.nrad = 0;
@@ -176,7 +178,7 @@ inline void make_plan(int M, FftPlan& p, bool big = true) {
   if (big)
     for (int r : {15, 13, 11, 9, 7, 5, 3, 8, 4, 2}) pull(m, r);
   else
-    for (int r : {5, 3, 7, 11, 13}) pull(m, r);
+    for (int r : {5, 3, 7, 11, 13, 8, 4, 2}) pull(m, r);
   for (int r = 17; m > 1; r += 2) {
     if ((long long)r * r > m) r = m;   // what is left is prime
     while (m % r == 0 && p.nrad < kMaxRadices) { p.radix[p.nrad++] = r; m /= r; }

@@ -135,3 +135,23 @@ def test_default_batch_launch_matches_one_cta_a_cell(hb, solver, cells):
     for i in range(cells):
         for key in ("upper", "lower"):
             assert np.abs(base[key][i] - one[key][i]).max() <= 1e-10 * np.linalg.norm(one[key][i]), (i, key)
+
+
+@pytest.mark.parametrize("N", [(16, 16), (48, 32), (80, 13), (64, 96), (16, 12, 32)])
+@pytest.mark.parametrize("arith", [0, 2])
+def test_mixed_gani_on_grids_with_powers_of_two(hb, solver, N, arith):
+    """GaNi transforms as long as an even grid, whose float-float residuals have factors 16 and
+    more: the FP64 solve to 1e-6 (the bar of the mixed GaNi tests), by default and with every
+    residual in float-float."""
+    d = len(N)
+    p = ms.make_problem(d, N, 1.0, 1.0, [ms.box((0.1, 0.05, 0.0)[:d], (0.3, 0.2, 0.5)[:d], 20.0, d),
+                                         ms.ball((-0.25, -0.2, 0.1)[:d], 0.12, 0.2, d)])
+    ref = solver(p, precision=hb.HOM_FP64, tol=1e-9, discretization=1)
+    hb.binding.hom_set_refine_arith(solver.ctx, arith)
+    try:
+        out = solver(p, precision=hb.HOM_MIXED, tol=1e-7, discretization=1)
+    finally:
+        hb.binding.hom_set_refine_arith(solver.ctx, 0)
+    assert out["status"] == 0
+    for key in ("gani_A", "gani_B", "upper", "lower"):
+        assert np.abs(out[key] - ref[key]).max() <= 1e-6 * np.linalg.norm(ref[key]), key
