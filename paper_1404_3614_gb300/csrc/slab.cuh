@@ -204,7 +204,8 @@ __device__ __forceinline__ void slab_twiddle(fpair2* v, const float2* Wt, int l,
   }
 }
 // Transpose of a lane group's R x R values through its pencil of shared memory: v[k] of lane l
-// goes to v[l] of lane k (own = false: nothing written, the values read are not used)
+// goes to v[l] of lane k (own = false: nothing written, the values read are not used; S is then
+// the pencil of another lane group of the same warp, which its barriers keep apart from writes)
 template <int R>
 __device__ __forceinline__ void slab_exchange(fpair2* v, fpair2* S, int l, bool own) {
   __syncwarp();
@@ -302,14 +303,17 @@ __global__ void __launch_bounds__(kSlabMaxThreads) k_slab(SlabArgs a) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarp = blockDim.x >> 5;
   // R = 15: one lane group to each half warp (the hardware serves a 64-bit access half by half:
   // groups on lanes 0-14 and 15-29 cost a third wavefront); else R lanes after one another
-  const int sub = R == 15 ? lane >> 4 : lane / R;
+  // Lanes outside a group (act = false) read what lane 0 of their warp's last group, or of their half
+  // warp, reads, and groups past the last pencil or rows (on = false) the last ones, which are
+  // their own warp's then: no warp reads what another one writes, and no access needs a predicate.
+  const int sub = R == 15 ? lane >> 4 : min(lane / R, PW - 1);
   const int l0 = R == 15 ? sub << 4 : sub * R;
-  const bool act = sub < PW && lane - l0 < R;
+  const bool act = lane - l0 < R;
   const int l = act ? lane - l0 : 0;
   const int lc = l > 0 ? R - l : 0;                      // the column of this lane's negative frequencies
   const int mirror = act && l > 0 ? l0 + lc : lane;      // and the lane that holds them
   const int slots = nwarp * PW;
-  const int slot = act ? warp * PW + sub : 0;
+  const int slot = warp * PW + sub;
   constexpr int nquad = (M + 3) / 4;     // groups of four rows (the last one holds M mod 4 = 1)
   static_assert(M % 4 == 1, "rows of the last group");
   fpair2* Sw = reinterpret_cast<fpair2*>(S) + (size_t)slot * M;
@@ -337,12 +341,12 @@ __global__ void __launch_bounds__(kSlabMaxThreads) k_slab(SlabArgs a) {
     // slab (row-major [Ny][Nh]), zero padded to M; columns past Nh are zero
     for (int c0 = 0; c0 < NC; c0 += slots) {
       if (c0 + warp * PW >= NC) break;   // no pair for this warp in this or a later round
-      const int c = c0 + slot;
-      const bool on = act && c < NC;
+      const int c = min(c0 + slot, NC - 1);
+      const bool on = act && c0 + slot < NC;
       const int mp = c / R;              // columns l' + R 2 mp and l' + R (2 mp + 1), l' = c mod R
       const int ka = c - mp * R + 2 * R * mp, kb = ka + R;
       const bool ona = on && ka < Nh, onb = on && kb < Nh;
-      fpair2* p = P + (size_t)(on ? c : 0) * LD;
+      fpair2* p = P + (size_t)c * LD;
       fpair2 v[R];
 #pragma unroll
       for (int n = 0; n < R; ++n) {
@@ -372,7 +376,7 @@ __global__ void __launch_bounds__(kSlabMaxThreads) k_slab(SlabArgs a) {
     for (int q0 = 0; q0 < nquad; q0 += slots) {
       if (q0 + warp * PW >= nquad) break;   // no rows for this warp
       const bool on = act && q0 + slot < nquad;
-      const int y0 = on ? 4 * (q0 + slot) : 0;
+      const int y0 = 4 * min(q0 + slot, nquad - 1);
       const bool four = y0 + 3 < M;         // else one row
       fpair2 v[R];
       {
@@ -495,7 +499,7 @@ __global__ void __launch_bounds__(kSlabMaxThreads) k_slab(SlabArgs a) {
     for (int c0 = 0; c0 < NC; c0 += slots) {
       if (c0 + warp * PW >= NC) break;
       const bool on = act && c0 + slot < NC;
-      fpair2* p = P + (size_t)(on ? c0 + slot : 0) * LD;
+      fpair2* p = P + (size_t)min(c0 + slot, NC - 1) * LD;
       fpair2 v[R];
 #pragma unroll
       for (int n = 0; n < R; ++n) v[n] = p[l + R * n];
