@@ -497,9 +497,9 @@ hom_status hom_set_pass_chunks(hom_ctx* ctx, int32_t ypass_pencils, int32_t xpas
  * forward y transforms into one pass over (rhs, component, z) slabs held in shared memory,
  * by persistent CTAs that stage each slab's input with a bulk asynchronous copy issued
  * while the previous slab is still being transformed (enable = 1, the default: warps per
- * CTA chosen from the slab's shape; 4..20 in steps of 4 asks for that many warps where they
- * fit, at most 15, and leaves the automatic choice where they do not). enable = 0 runs them as three separate passes; the results agree to
- * rounding. A staged copy that does not complete within a bounded wait makes hom_bounds
+ * CTA chosen from the slab's shape; 4..20 in steps of 4 asks for that many warps, and leaves
+ * the automatic choice where their shared memory does not fit: 20 at M = 225). enable = 0 runs
+ * them as three separate passes; the results agree to rounding. A staged copy that does not complete within a bounded wait makes hom_bounds
  * return HOM_ERR_TIMEOUT. Applies to later calls on this context. */
 hom_status hom_set_slab_pass(hom_ctx* ctx, int32_t enable);
 /* The first and last passes of the FP32 3D operator at double-grid length 225 along z

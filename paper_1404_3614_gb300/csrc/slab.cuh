@@ -23,7 +23,10 @@
 
 namespace homb {
 
-constexpr int kSlabMaxThreads = 480;   // 15 warps: up to 136 registers a thread
+// 16 warps at 128 registers a thread (what the kernel takes), and, at a caller's request for more,
+// 20 warps at 96 in a compilation of their own (R < 15: 20 warps' scratch at 225 exceeds the
+// shared memory)
+constexpr int kSlabMaxThreads = 512, kSlabWideThreads = 640;
 
 // Layout of the slab in shared memory: columns kx = l + R m and l + R (m + 1), m even, side by side
 // (a column pair: one lane group's two pencils in the y passes, and two of a lane's values
@@ -225,8 +228,8 @@ __device__ __forceinline__ fpair slab_shfl(fpair a, int src) {
 // pencil a lane group: 259 M -> 126 M warp instructions. It is bound by shared-memory
 // accesses now (72 % of the L1 data pipe; FP32 pipe 45 %, issue 39 %): a pencil passes through
 // shared memory once between its two register DFTs, and once between the y and x passes.
-template <int R, bool ZB>
-__global__ void __launch_bounds__(kSlabMaxThreads) k_slab(SlabArgs a) {
+template <int R, bool ZB, int NT = kSlabMaxThreads>
+__global__ void __launch_bounds__(NT) k_slab(SlabArgs a) {
   using F = fpair;
   constexpr int M = R * R;
   constexpr int LD = slab_ld(M);
@@ -532,22 +535,29 @@ __global__ void __launch_bounds__(kSlabMaxThreads) k_slab(SlabArgs a) {
   }
 }
 
-template <int R, bool ZB> cudaError_t launch_slab_rz(const SlabArgs& a, int warps, cudaStream_t s) {
+template <int R, bool ZB, int NT> cudaError_t launch_slab_nt(const SlabArgs& a, int warps, cudaStream_t s) {
   const size_t smem = slab_smem_bytes(R, ZB, a.Ny, a.Nh, warps);
   static std::atomic<int> cache[kAttrDevices] = {};
-  cudaError_t e = smem_attr(k_slab<R, ZB>, smem, cache);
+  cudaError_t e = smem_attr(k_slab<R, ZB, NT>, smem, cache);
   if (e != cudaSuccess) return e;
   // persistent: as many CTAs as are resident at once, at most one per slab
   int dev = 0, sms = 0, per = 0;
   e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_slab<R, ZB>, warps * 32, smem);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_slab<R, ZB, NT>, warps * 32, smem);
   if (e != cudaSuccess) return e;
   if (per < 1) return cudaErrorInvalidConfiguration;
   const long long nslabs = (long long)a.nrc * a.Mz;
   const int grid = (int)std::min<long long>(nslabs, (long long)sms * per);
-  k_slab<R, ZB><<<grid, warps * 32, smem, s>>>(a);
+  k_slab<R, ZB, NT><<<grid, warps * 32, smem, s>>>(a);
   return cudaGetLastError();
+}
+
+template <int R, bool ZB> cudaError_t launch_slab_rz(const SlabArgs& a, int warps, cudaStream_t s) {
+  if constexpr (R < 15) {
+    if (warps * 32 > kSlabMaxThreads) return launch_slab_nt<R, ZB, kSlabWideThreads>(a, warps, s);
+  }
+  return launch_slab_nt<R, ZB, kSlabMaxThreads>(a, warps, s);
 }
 
 // The zero band applies when the y rows (Ny stored around 0) and the Hermitian x extension
@@ -593,17 +603,21 @@ template <typename T> int slab_warps(int M, int Ny, int Nh) {
   return best;
 }
 
+// The same with a caller's choice of warps (0: none), taken where it fits
+template <typename T> int slab_warps_asked(int M, int Ny, int Nh, int asked) {
+  const int warps = slab_warps<T>(M, Ny, Nh);
+  if (warps == 0 || asked <= 0) return warps;
+  const int r = M == 225 ? 15 : (M == 81 ? 9 : (M == 25 ? 5 : 3));
+  const bool fits = asked * 32 <= (r < 15 ? kSlabWideThreads : kSlabMaxThreads) &&
+                    slab_smem_bytes(r, slab_band_free(M, Ny, Nh), Ny, Nh, asked) <= 227 * 1024;
+  return fits ? asked : warps;
+}
+
 template <typename T> cudaError_t launch_slab(const SlabArgs& a, cudaStream_t s) {
   if constexpr (sizeof(T) != 4) {
     return cudaErrorNotSupported;
   } else {
-    int warps = slab_warps<T>(a.M, a.Ny, a.Nh);
-    if (warps && a.warps > 0) {   // a caller's choice, where it fits
-      const int r = a.M == 225 ? 15 : (a.M == 81 ? 9 : (a.M == 25 ? 5 : 3));
-      const bool zb = slab_band_free(a.M, a.Ny, a.Nh);
-      if (a.warps * 32 <= kSlabMaxThreads && slab_smem_bytes(r, zb, a.Ny, a.Nh, a.warps) <= 220 * 1024)
-        warps = a.warps;
-    }
+    const int warps = slab_warps_asked<T>(a.M, a.Ny, a.Nh, a.warps);
     switch (warps ? a.M : 0) {
       case 9: return launch_slab_r<3>(a, warps, s);
       case 25: return launch_slab_r<5>(a, warps, s);

@@ -155,3 +155,28 @@ def test_mixed_gani_on_grids_with_powers_of_two(hb, solver, N, arith):
     assert out["status"] == 0
     for key in ("gani_A", "gani_B", "upper", "lower"):
         assert np.abs(out[key] - ref[key]).max() <= 1e-6 * np.linalg.norm(ref[key]), key
+
+
+@pytest.mark.parametrize("N", [5, 13, 41, 113])
+def test_slab_pass_warp_counts(hb, solver, N):
+    """Every count of warps a CTA that can be asked for (at M = 225 the automatic one in place of 20)
+    computes the operator of the separate passes: 2e-6 of the largest entry, the bar of the slab test."""
+    p = ms.random_spheres_3d(7, N=N, n_balls=5, phi=0.2, contrast=100.0)
+    info = hb.hom_problem_info(solver.ctx, p)
+    nws = hb.hom_step_workspace_size(solver.ctx, p, 3)
+    ws = torch.empty(nws, dtype=torch.uint8, device="cuda")
+    coef = torch.empty((info["ncomp"],) + tuple(info["M"][::-1]), dtype=torch.float32, device="cuda")
+    hb.hom_coefficient(solver.ctx, p, 0, hb.HOM_FP32, coef.data_ptr(), ws.data_ptr(), nws)
+    x = torch.randn((3, 3, N, N, (N + 1) // 2), generator=torch.Generator().manual_seed(N), dtype=torch.complex64).cuda()
+    out = {}
+    try:
+        for slab in (0, 1, 4, 8, 12, 16, 20):
+            hb.hom_set_slab_pass(solver.ctx, slab)
+            y = torch.zeros_like(x)
+            hb.hom_matvec(solver.ctx, p, 0, hb.HOM_FP32, 1, 3, coef.data_ptr(), x.data_ptr(), y.data_ptr(), ws.data_ptr(), nws)
+            torch.cuda.synchronize()
+            out[slab] = y
+    finally:
+        hb.hom_set_slab_pass(solver.ctx, 1)
+    for slab, y in out.items():
+        assert (y - out[0]).abs().max() <= 2e-6 * out[0].abs().max(), slab

@@ -94,8 +94,13 @@ template <typename T> static std::vector<T> load(const char* f) {
   std::fclose(h);
   return v;
 }
-// M N nrc Mz warps in coef twiddles out
+// M N nrc Mz warps in coef twiddles out; or M N asked: the warps of a launch
 int main(int argc, char** argv) {
+  if (argc == 4) {
+    const int M = std::atoi(argv[1]), N = std::atoi(argv[2]);
+    std::printf("%d\n", slab_warps_asked<float>(M, N, (N + 1) / 2, std::atoi(argv[3])));
+    return 0;
+  }
   const int M = std::atoi(argv[1]), N = std::atoi(argv[2]), nrc = std::atoi(argv[3]), Mz = std::atoi(argv[4]);
   int warps = std::atoi(argv[5]);
   std::vector<float2> x = load<float2>(argv[6]), W = load<float2>(argv[8]);
@@ -142,7 +147,7 @@ def host_slab_source():
     """The kernel, its layout and its size rules, with the PTX statements taken out (the bulk copy: a
     plain one)."""
     src = open(os.path.join(CSRC, "slab.cuh")).read()
-    kern = src[src.index("constexpr int kSlabMaxThreads"):src.index("template <int R, bool ZB> cudaError_t launch_slab_rz")]
+    kern = src[src.index("constexpr int kSlabMaxThreads"):src.index("template <int R, bool ZB, int NT> cudaError_t launch_slab_nt")]
     rules = src[src.index("inline bool slab_band_free"):src.index("template <int R> cudaError_t launch_slab_r")]
     rules += src[src.index("template <typename T> int slab_warps"):src.index("template <typename T> cudaError_t launch_slab(")]
     wait = kern.index("__device__ __forceinline__ bool slab_wait")
@@ -216,3 +221,15 @@ def test_slab_kernel(exe, tmp_path, M, N, warps):
     for rc in (0, 2):
         ref = reference(x[rc, 0].astype(complex), coef[0].astype(float), M, N)
         assert np.abs(y[rc, 0] - ref).max() <= 1e-5 * np.abs(ref).max()
+
+
+def warps_of(exe, M, N, asked):
+    return int(subprocess.run([str(exe), str(M), str(N), str(asked)], check=True, capture_output=True, text=True).stdout)
+
+
+@pytest.mark.parametrize("M,N", [(9, 5), (25, 13), (81, 41), (225, 113), (9, 9), (25, 25), (81, 81)])
+def test_asked_warps_are_taken_where_they_fit(exe, M, N):
+    auto = warps_of(exe, M, N, 0)
+    assert auto > 0
+    for asked in (4, 8, 12, 16, 20):
+        assert warps_of(exe, M, N, asked) == (auto if (M, asked) == (225, 20) else asked)
