@@ -529,9 +529,9 @@ __device__ __forceinline__ void xpass_warp(const XArgs& a, cpx<T>* Ws, cpx<T>* A
 // copy. Bound by issue and shared memory; with 3 x 3 fields, N = 51 (99225 rows of 105 points) 85 ->
 // 81 us against one pair a pencil, N = 79 (primes in 157) 98 -> 80 us the whole operator, mixed 2D and
 // 3D bounds 2 to 25 % faster.
-constexpr int kXPairThreads = 128;
+constexpr int kXPairThreads = 128, kXPairMaxThreads = 256;
 template <int MT>
-__global__ void __launch_bounds__(kXPairThreads, 4) k_xpass_pair(XArgs a) {
+__global__ void __launch_bounds__(kXPairMaxThreads, 2) k_xpass_pair(XArgs a) {
   using F = fpair;
   extern __shared__ __align__(16) unsigned char smem[];
   const int M = MT > 0 ? MT : a.M;
@@ -927,27 +927,44 @@ template <typename T, int MT> cudaError_t launch_final_m(FinalArgs a, cudaStream
 
 // shared memory of the packed row pass: duplicated twiddles and two buffers of double pencils
 inline size_t xpair_smem(int M, int nrow) { return (size_t)M * 16 * (1 + 2 * (size_t)((nrow + 3) / 4)); }
-// planes per CTA: as many double pencils as 48 KB hold (four CTAs an SM), whole groups of four rows
-// where they fit; 0 where one plane exceeds the shared memory
-inline int xpair_yb(int M, int rpp, int planes, int gy) {
-  if (xpair_smem(M, rpp) > kPassSmemMax) return 0;
-  long long yb = 1;
-  while (yb < 32 && yb < planes && xpair_smem(M, (int)(yb + 1) * rpp) <= kPassSmemBudget) ++yb;
-  yb = spread_chunk(yb, planes, gy);
+// Planes and threads of its CTAs; yb = 0: k_xpass runs instead. As many double pencils as 48 KB hold
+// (four CTAs an SM), while they hold a whole group of rows: two planes of two rows in one double
+// pencil (2D, M <= 1024), four planes of three in three (3D, M <= 438). Longer:
+//  - k_xpass where 48 KB hold two planes of three rows, three pairs (3D, M <= 877): at M = 621, 729
+//    and 809 59, 118 and 456 us the anisotropic operator; 69, 135 and 704 with double pencils left
+//    partly empty, 61, 127 and 473 with 110 KB;
+//  - else 110 KB, two CTAs an SM of twice the threads. Two planes share a double pencil however long it is;
+//    one plane alone left half of it empty (2D, M = 1025, 1401, 2049: 101, 447 and 1360 us the
+//    operator for 132, 711 and 2486 so; 112, 538 and 1461 with k_xpass);
+//  - k_xpass where 110 KB hold no double pencil (M > 2346: at M = 2693 9.0 ms for 9.8 with one CTA an SM)
+//    or a CTA gets a single pair of rows.
+constexpr size_t kXPairSmemLong = 110 * 1024;
+struct XPairShape {
+  int yb, threads;
+};
+inline XPairShape xpair_shape(int M, int rpp, int planes, int gy) {
+  auto pencils = [M](size_t smem) { return ((long long)(smem / ((size_t)M * 16)) - 1) / 2; };
+  const bool small = pencils(kPassSmemBudget) >= (rpp == 3 ? 3 : 1);
+  if (!small && rpp == 3 && (size_t)M * 8 * 7 <= kPassSmemBudget) return {0, 0};
+  const long long n = pencils(small ? kPassSmemBudget : kXPairSmemLong);
+  if (n < 1) return {0, 0};
+  long long yb = spread_chunk(std::min<long long>(std::min(32, planes), 4 * n / rpp), planes, gy);
   while (yb > 1 && (yb * rpp) % 4 != 0 && ((yb - 1) * rpp) % 4 == 0) --yb;
-  return (int)yb;
+  if (!small && yb * rpp <= 2) return {0, 0};
+  return {(int)yb, small ? kXPairThreads : pass_threads((int)((yb * rpp + 3) / 4), M, false)};
 }
 
 template <typename T, int MT> cudaError_t launch_xpass_m(XArgs a, int grid_y, cudaStream_t s) {
   if constexpr (sizeof(T) == 4) {
-    const int yb = a.mode == 0 && a.pair ? xpair_yb(a.M, a.C, a.planes, grid_y) : 0;
+    const XPairShape x = a.mode == 0 && a.pair ? xpair_shape(a.M, a.C, a.planes, grid_y) : XPairShape{0, 0};
+    const int yb = x.yb;
     if (yb > 0) {
       a.YB = yb;
       const size_t smem = xpair_smem(a.M, yb * a.C);
       static std::atomic<int> pcache[kAttrDevices] = {};
       const cudaError_t e = smem_attr(k_xpass_pair<MT>, smem, pcache);
       if (e != cudaSuccess) return e;
-      k_xpass_pair<MT><<<dim3((a.planes + yb - 1) / yb, grid_y), kXPairThreads, smem, s>>>(a);
+      k_xpass_pair<MT><<<dim3((a.planes + yb - 1) / yb, grid_y), x.threads, smem, s>>>(a);
       return cudaGetLastError();
     }
   }

@@ -180,3 +180,31 @@ def test_slab_pass_warp_counts(hb, solver, N):
         hb.hom_set_slab_pass(solver.ctx, 1)
     for slab, y in out.items():
         assert (y - out[0]).abs().max() <= 2e-6 * out[0].abs().max(), slab
+
+
+# the packed row pass past 48 KB: two planes a double pencil, three and four, a plane alone; the
+# unpacked one: a single pair of rows, no double pencil in 110 KB, three pairs of three rows
+@pytest.mark.parametrize("N,aniso", [((521, 81), True), ((521, 161), False), ((527, 305), True), ((521, 9), False),
+                                     ((1175, 5), True), ((1001, 79), False), ((221, 5, 5), True), ((405, 3, 5), False),
+                                     ((441, 5, 3), True), ((441, 9, 9), True), ((527, 9, 7), False)])
+def test_long_rows_match_oracle(hb, solver, N, aniso):
+    """FP32 operator: 5e-6 of the largest entry, the bar of the operator's step tests."""
+    d = len(N)
+    A0, A1 = (((A2, A2 @ A2) if d == 2 else (A3, A3 @ A3)) if aniso else (1.0, 20.0))
+    p = ms.make_problem(d, N, (1.0, 0.7, 1.2)[:d], A0, [ms.box((0.1, 0.05, 0.0)[:d], (0.3, 0.2, 0.5)[:d], A1, d),
+                                                        ms.ball((-0.25, -0.2, 0.1)[:d], 0.12, 0.2, d)])
+    rng = np.random.default_rng([zlib.crc32(b"long"), *N])
+    op = matfree.MatFreeOperator(p, "primal")
+    info = hb.hom_problem_info(solver.ctx, p)
+    nws = hb.hom_step_workspace_size(solver.ctx, p, d)
+    ws = torch.empty(nws, dtype=torch.uint8, device="cuda")
+    fields = [random_real_field(rng, d, N) for _ in range(d)]
+    ref = np.stack([full_to_half(op.apply(u, project=True), d) for u in fields])
+    x = torch.from_numpy(np.stack([full_to_half(u, d) for u in fields]).astype(np.complex64)).cuda()
+    coef = torch.empty((info["ncomp"],) + tuple(info["M"][:d][::-1]), dtype=torch.float32, device="cuda")
+    hb.hom_coefficient(solver.ctx, p, 0, hb.HOM_FP32, coef.data_ptr(), ws.data_ptr(), nws)
+    y = torch.zeros_like(x)
+    hb.hom_matvec(solver.ctx, p, 0, hb.HOM_FP32, 1, d, coef.data_ptr(), x.data_ptr(), y.data_ptr(), ws.data_ptr(), nws)
+    torch.cuda.synchronize()
+    scale = max(np.abs(ref).max(), x.abs().max().item())
+    assert np.abs(y.cpu().numpy() - ref).max() < 5e-6 * scale
