@@ -61,4 +61,4 @@ def test_rows_fill_their_double_pencils(shapes):
             assert yb % 2 == 0, M
         else:
             assert (yb > 0) == (M <= 438 or 877 < M <= 2346), M
-            assert yb >= 4 or M > 877, M   # four planes are three whole groups
+            assert yb >= 4 or M > 438, M   # four planes are three whole groups
