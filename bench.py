@@ -708,7 +708,8 @@ def batched_timings(hb, solver, dev, n=256, reps=3, autotune=1):
             e0 = torch.cuda.Event(enable_timing=True)
             e1 = torch.cuda.Event(enable_timing=True)
             e0.record(stream)
-        out = solver.batched(probs, precision=hb.HOM_MIXED, tol=TOL, graph=1, stream=stream.cuda_stream)
+        out = solver.batched(probs, precision=hb.HOM_MIXED, tol=TOL, autotune=autotune, graph=1,
+                             stream=stream.cuda_stream)
         with torch.cuda.stream(stream):
             e1.record(stream)
         e1.synchronize()

@@ -164,8 +164,11 @@ typedef struct {
                            iterations from captured CUDA graphs, -1 launches every
                            kernel directly; hom_bounds_batched: 1 replays the batch
                            launch as a graph captured on `stream` (non-NULL)     */
-  int32_t autotune;     /* hom_bounds_batched: time the shared-memory chunk sizes
-                           on this batch once and keep the fastest in the ctx    */
+  int32_t autotune;     /* hom_bounds_batched: time launch configurations (the untuned
+                           one among them) on this batch once and keep the fastest
+                           in the ctx, for later calls that set it, of the same
+                           largest grid and precision and about as many cells. Calls
+                           without it do not depend on it.                        */
   int32_t dual_start;   /* hom_bounds with both sides: 0 starts the dual CG from
                            zero; 1 starts it from the primal minimisers (Remark
                            "Avoiding the solution of dual formulation", Eq.
@@ -542,7 +545,7 @@ hom_status hom_set_refine_arith(hom_ctx* ctx, int32_t mode);
 
 /* Threads per CTA of the persistent batched kernel: 256 (two CTAs per SM), 512 or 1024
  * (one CTA per SM: more threads per cell, fewer cells at a time), or 0 (default: the
- * autotuned choice when hom_opts.autotune is set, else by the batch's cell sizes; 256 when
+ * autotuned choice when hom_opts.autotune is set, else by the batch's cells; 256 when
  * hom_set_batch_cluster chose a cluster). Applies to later hom_bounds_batched calls on this
  * context. */
 hom_status hom_set_batch_threads(hom_ctx* ctx, int32_t threads);

@@ -2130,7 +2130,9 @@ hom_status hom_bounds_batched(hom_ctx* ctx, int32_t n, const hom_problem* probs,
     const int g_ = std::min(bp.nslots_max, mx);
     return (g_ / cluster) * cluster;
   };
-  int run_stride = 0;
+  // launches that the library chooses, tuned or not, round |r|^2 alike; a caller's own keep the
+  // grouping of their team
+  const int run_stride = ctx->batch_threads || ctx->batch_cluster ? 0 : 256;
   int launched[6] = {0, 0, 0, 0, 0, 0};   // threads, cap, schedule, cluster, coopM, CTAs
   auto enqueue = [&](int cap, int threads, int cluster, int coopM, int max_iter) -> hom_status {
     size_t smem = 0;
@@ -2157,19 +2159,41 @@ hom_status hom_bounds_batched(hom_ctx* ctx, int32_t n, const hom_problem* probs,
     CK(d2h_copy(ctx, ctx->pin_out, base + bp.o_energy, bp.out_bytes, st));
     return HOM_OK;
   };
-  // chunk capacity and threads per CTA: autotuned once per (grid extent, precision), or
-  // the defaults; a thread count set on the context overrides both
-  int cap = std::max(2048, cap_min);
+  // chunk capacity, threads per CTA and clusters: for calls that ask for it, autotuned once per
+  // (grid extent, precision, power of two of tasks), else by the batch's sizes; a thread count or
+  // cluster set on the context overrides both
+  const int cap0 = std::max(2048, cap_min);
+  int cap = cap0;
   int threads = 256, sched = 0, cluster = 1, coopM = 0;
   // the radix schedule travels in the staged task table (both axes' plans of every task)
   auto set_sched = [&](int sc) {
     BTask* tk = reinterpret_cast<BTask*>(ctx->pin_in);
     for (long long k = 0; k < nt; ++k) tk[k].plan0.sched = tk[k].plan1.sched = sc;
   };
-  const long long tkey = ((long long)bp.Mmax * 4 + (f32 ? 1 : 0)) * 2 + ctx->batch_wpass;
+  // The launch without tuning: every task on a cluster of 8 CTAs, so that no long
+  // task is left alone on one SM while the others idle. CTAs of 512 threads (15 clusters at
+  // once) where the longest task is a large part of a cluster's share of the batch, else 256
+  // (36 clusters). Against one 256-thread CTA a task: 64 cells of mixed N 235 -> 32 ms (512;
+  // 43 with 256), 24 of them 182 -> 22, 200 of them 262 -> 64 (256; 75 with 512), 63 cells of
+  // N = 89 164 -> 43 (256; 45), 16 of N = 113 28.7 -> 5.5 (512; 6.4). Cells up to N = 32 have
+  // too little work for 8 CTAs: clusters of 4 (64 cells of N = 23: 7.5 -> 6.7 ms, 7.5 with 8).
+  auto default_launch = [&](int* th, int* cl) {
+    double work = 0.0, longest = 0.0;
+    for (const BTask& t : bp.tasks) {
+      const double w = (double)t.M0 * t.M1;
+      work += w;
+      longest = std::max(longest, w);
+    }
+    const int c = bp.Mmax <= 64 ? 4 : 8;
+    size_t sm_ = 0;
+    const int clusters = grid_for(cap0, 256, c, &sm_, c > 1) / c;
+    *cl = c;
+    *th = c == 8 && work < 2.0 * clusters * longest ? 512 : 256;
+  };
+  const long long tkey = (((long long)bp.Mmax * 4 + (f32 ? 1 : 0)) * 2 + ctx->batch_wpass) * 64 + std::ilogb((double)nt);
   bool tuned = false;
   for (auto& kv : ctx->tuned_cap)
-    if (kv.key == tkey) {
+    if (opts->autotune && kv.key == tkey) {
       cap = std::max(kv.cap, cap_min);
       threads = kv.threads;
       sched = kv.sched;
@@ -2203,55 +2227,55 @@ hom_status hom_bounds_batched(hom_ctx* ctx, int32_t n, const hom_problem* probs,
     threads = best_threads;
     sched = best_sched;
     set_sched(sched);
-    // clusters for the largest cells: timed on whole solves of this batch, since they act
-    // on the longest tasks at the end of the launch, which short probes do not see
+    // clusters for the largest cells, and the launches of every cell on clusters, the untuned one
+    // among them: timed on whole solves of this batch, since they act on the longest tasks at the
+    // end of the launch, which short probes do not see
     const int mtop = std::max(bp.tasks[0].M0, bp.tasks[0].M1);
     int msecond = 0;
     for (const BTask& tk : bp.tasks)
       if (std::max(tk.M0, tk.M1) < mtop) { msecond = std::max(tk.M0, tk.M1); break; }
     best = 1e30f;
     const int solve_iter = opts->max_iter > 0 ? opts->max_iter : 10000;
-    struct Cand { int cl, m; };
-    std::vector<Cand> cands = {{1, 0}, {2, mtop}, {4, mtop}, {8, mtop}};
+    std::vector<hom_ctx::Tuned> cands;   // the first one wins a tie
+    auto cand = [&](int cap_, int th, int sc, int cl, int m) { cands.push_back({tkey, cap_, th, sc, cl, m}); };
+    int th0 = 256, cl0 = 1;
+    default_launch(&th0, &cl0);
+    cand(cap0, th0, 0, cl0, 0);
+    for (int cl : {1, 2, 4, 8}) cand(cap, threads, sched, cl, cl > 1 ? mtop : 0);
     if (msecond > 0) {
-      cands.push_back({4, msecond});
-      cands.push_back({8, msecond});
+      cand(cap, threads, sched, 4, msecond);
+      cand(cap, threads, sched, 8, msecond);
     }
-    for (const Cand& cd : cands) {
+    for (int th : {256, 512})
+      for (int cl : {4, 8})
+        if (th != th0 || cl != cl0) cand(cap0, th, 0, cl, 0);
+    hom_ctx::Tuned pick = cands[0];
+    for (const hom_ctx::Tuned& cd : cands) {
       size_t sm_ = 0;
-      if (cd.cl > 1 && grid_for(cap, threads, cd.cl, &sm_) < cd.cl) continue;
+      if (cd.cluster > 1 && grid_for(cd.cap, cd.threads, cd.cluster, &sm_, ncoop_for(cd.cluster, cd.coopM) == nt) < cd.cluster)
+        continue;
+      set_sched(cd.sched);
+      CKS(enqueue(cd.cap, cd.threads, cd.cluster, cd.coopM, 3));   // untimed: loads the kernel
       CK(cudaEventRecord(e0, st));
-      CKS(enqueue(cap, threads, cd.cl, cd.m, solve_iter));
+      CKS(enqueue(cd.cap, cd.threads, cd.cluster, cd.coopM, solve_iter));
       CK(cudaEventRecord(e1, st));
       CK(cudaEventSynchronize(e1));
       float ms = 0;
       CK(cudaEventElapsedTime(&ms, e0, e1));
-      if (ms < best) { best = ms; cluster = cd.cl; coopM = cd.m; }
+      if (ms < best) { best = ms; pick = cd; }
     }
+    cap = pick.cap;
+    threads = pick.threads;
+    sched = pick.sched;
+    cluster = pick.cluster;
+    coopM = pick.coopM;
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    ctx->tuned_cap.push_back({tkey, cap, threads, sched, cluster, coopM});
+    ctx->tuned_cap.push_back(pick);
   }
   if (!tuned && !opts->autotune && ctx->batch_threads == 0 && ctx->batch_cluster == 0) {
-    // Neither tuned nor chosen by the caller: every task on a cluster of 8 CTAs, so that no long
-    // task is left alone on one SM while the others idle. CTAs of 512 threads (15 clusters at
-    // once) where the longest task is a large part of a cluster's share of the batch, else 256
-    // (36 clusters). Against one 256-thread CTA a task: 64 cells of mixed N 235 -> 32 ms (512;
-    // 43 with 256), 24 of them 182 -> 22, 200 of them 262 -> 64 (256; 75 with 512), 63 cells of
-    // N = 89 164 -> 43 (256; 45), 16 of N = 113 28.7 -> 5.5 (512; 6.4). Cells up to N = 32 have
-    // too little work for 8 CTAs: clusters of 4 (64 cells of N = 23: 7.5 -> 6.7 ms, 7.5 with 8).
-    double work = 0.0, longest = 0.0;
-    for (const BTask& t : bp.tasks) {
-      const double w = (double)t.M0 * t.M1;
-      work += w;
-      longest = std::max(longest, w);
-    }
-    cluster = bp.Mmax <= 64 ? 4 : 8;
+    default_launch(&threads, &cluster);
     coopM = 0;
-    size_t sm_ = 0;
-    const int clusters = grid_for(cap, 256, cluster, &sm_, true) / cluster;
-    threads = cluster == 8 && work < 2.0 * clusters * longest ? 512 : 256;
-    run_stride = 256;
   }
   set_sched(sched);
   if (ctx->batch_threads) threads = ctx->batch_threads;

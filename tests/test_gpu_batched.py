@@ -198,3 +198,22 @@ def test_warp_passes_match_block_passes(hb, solver, cluster, threads):
         hb.binding.hom_set_batch_warp_passes(solver.ctx, 1)
         hb.binding.hom_set_batch_threads(solver.ctx, 0)
         hb.binding.hom_set_batch_cluster(solver.ctx, 0, 0)
+
+
+def test_plain_calls_do_not_depend_on_tuned_ones(hb):
+    """A call without autotune launches the same and returns the same bits before and after a tuned call
+    on its context; a later tuned call of the same batch takes the tuned launch again."""
+    probs = [ms.random_rectangles_2d(s + 200, N=(63, 23)[s % 2]) for s in range(10)]
+    s = hb.Bounds(0)
+    try:
+        for prec in (hb.HOM_MIXED, hb.HOM_FP64):
+            before = s.batched(probs, precision=prec, tol=1e-4)
+            tuned = s.batched(probs, precision=prec, tol=1e-4, autotune=1)
+            after = s.batched(probs, precision=prec, tol=1e-4)
+            again = s.batched(probs, precision=prec, tol=1e-4, autotune=1)
+            assert after["report"]["config"] == before["report"]["config"]
+            assert np.array_equal(after["upper"], before["upper"]) and np.array_equal(after["lower"], before["lower"])
+            assert again["report"]["config"] == tuned["report"]["config"]
+            assert np.array_equal(again["upper"], tuned["upper"])
+    finally:
+        s.close()
