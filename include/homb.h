@@ -554,8 +554,8 @@ hom_status hom_set_batch_threads(hom_ctx* ctx, int32_t threads);
  * double-grid extent 2N-1 is at least coop_min_M are each worked on by all `cluster` CTAs
  * of a cluster together (splitting every transform pass and reduction over them, with
  * cluster barriers between passes); the other cells take one CTA each. cluster 1 turns
- * this off; 0 (default) uses the autotuned choice when hom_opts.autotune is set, else 4 or 8 for
- * every cell (1 when hom_set_batch_threads chose a CTA size).
+ * this off; 0 (default) uses the autotuned choice when hom_opts.autotune is set, else 1, 2, 4 or 8 for
+ * every cell by the batch's sizes (1 when hom_set_batch_threads chose a CTA size).
  * Results equal the single-CTA ones to rounding (reduction order). Applies to later
  * hom_bounds_batched calls on this context. */
 hom_status hom_set_batch_cluster(hom_ctx* ctx, int32_t cluster, int32_t coop_min_M);

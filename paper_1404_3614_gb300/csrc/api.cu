@@ -2170,13 +2170,21 @@ hom_status hom_bounds_batched(hom_ctx* ctx, int32_t n, const hom_problem* probs,
     BTask* tk = reinterpret_cast<BTask*>(ctx->pin_in);
     for (long long k = 0; k < nt; ++k) tk[k].plan0.sched = tk[k].plan1.sched = sc;
   };
-  // The launch without tuning: every task on a cluster of 8 CTAs, so that no long
-  // task is left alone on one SM while the others idle. CTAs of 512 threads (15 clusters at
-  // once) where the longest task is a large part of a cluster's share of the batch, else 256
-  // (36 clusters). Against one 256-thread CTA a task: 64 cells of mixed N 235 -> 32 ms (512;
-  // 43 with 256), 24 of them 182 -> 22, 200 of them 262 -> 64 (256; 75 with 512), 63 cells of
-  // N = 89 164 -> 43 (256; 45), 16 of N = 113 28.7 -> 5.5 (512; 6.4). Cells up to N = 32 have
-  // too little work for 8 CTAs: clusters of 4 (64 cells of N = 23: 7.5 -> 6.7 ms, 7.5 with 8).
+  // The launch without tuning: every task on a cluster of CTAs, so that no long task is left alone
+  // on one SM while the others idle: 8, or 4 for cells up to N = 32, which have too little work
+  // for 8 (64 cells of N = 23: 7.5 -> 6.7 ms, 7.5 with 8). Fewer where the batch holds so many tasks
+  // that they fill the GPU by themselves: a cluster's barriers and ragged rounds then cost more than the
+  // long tasks' ends, the more so the smaller the cell (and less in FP64, whose pipe is shared by
+  // an SM). In tasks of the longest's size, clusters of 1 / 2 / 4 / 8 took (mixed, ms; * chosen):
+  //   23: 128 9.1 / 8.5 / 7.2* / 7.3;  256 11.2 / 10.8 / 10.5* / 12.4;  512 16.3 / 15.7* / 17.7 / 22.1;  2048 50* / 56 / 65 / 107
+  //   41: 256 28.1 / 21.7 / 20.9* / 22.3;  512 33.1 / 27.5* / 28.8 / 35.7;  2048 84.7* / 87.6 / 101 / 131
+  //   63: 64 31.6 / 18.6 / 11.6 / 8.0*;  512 52.2 / 37.4 / 34.9* / 37.6;  2048 132* / 117 / 119 / 138
+  //   113: 256 87 / 53 / 41 / 35*;  2048 250 / 216* / 208 / 220
+  // and FP64 23: 512 53.9 / 45.2 / 51.2* / 105;  2048 130* / 145 / 182 / 283;  63: 1024 581 / 464 / 395* / 403.
+  // CTAs of 512 threads (15 clusters of 8 at once) where the longest task is a large part of a
+  // cluster's share of the batch, else 256 (36 clusters): 64 cells of mixed N 235 ms with one CTA a task, 32
+  // (512), 41 (256), FP64 452 and 493; 256 of them 266, 92 and 68, FP64 1016 and 780; 63 cells of N = 89 147, 47 and
+  // 42, FP64 335 and 301; 16 of N = 113 60, 11.3 and 13.3, FP64 136 and 159.
   auto default_launch = [&](int* th, int* cl) {
     double work = 0.0, longest = 0.0;
     for (const BTask& t : bp.tasks) {
@@ -2184,7 +2192,8 @@ hom_status hom_bounds_batched(hom_ctx* ctx, int32_t n, const hom_problem* probs,
       work += w;
       longest = std::max(longest, w);
     }
-    const int c = bp.Mmax <= 64 ? 4 : 8;
+    int c = bp.Mmax <= 64 ? 4 : 8;
+    while (c > 1 && work * c > (f32 ? 24.0 : 48.0) * bp.Mmax * longest) c /= 2;
     size_t sm_ = 0;
     const int clusters = grid_for(cap0, 256, c, &sm_, c > 1) / c;
     *cl = c;

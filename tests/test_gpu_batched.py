@@ -200,6 +200,11 @@ def test_warp_passes_match_block_passes(hb, solver, cluster, threads):
         hb.binding.hom_set_batch_cluster(solver.ctx, 0, 0)
 
 
+def launch(out):
+    c = out["report"]["config"]
+    return c["threads"], c["cluster"]
+
+
 def test_plain_calls_do_not_depend_on_tuned_ones(hb):
     """A call without autotune launches the same and returns the same bits before and after a tuned call
     on its context; a later tuned call of the same batch takes the tuned launch again."""
@@ -217,3 +222,28 @@ def test_plain_calls_do_not_depend_on_tuned_ones(hb):
             assert np.array_equal(again["upper"], tuned["upper"])
     finally:
         s.close()
+
+
+# runs of |r|^2 that fill no 8 x 256 entries, ragged ones, and every launch the size rule picks
+@pytest.mark.parametrize("cells,N,want", [(3, 9, (256, 4)), (70, 9, (256, 2)), (160, 9, (256, 1)), (4, 41, (512, 8)),
+                                          (4, 113, (512, 8)), (40, 63, (256, 8))])
+@pytest.mark.parametrize("prec", ["mixed", "fp64"])
+def test_default_launches_match_one_cta_a_cell(hb, solver, cells, N, want, prec):
+    """Contrast 10 at tol 1e-5: a bound's error is the residual's energy, at most 10 tol^2 of the
+    bound for each solve: 1e-8 of 256-thread single CTAs, with a factor to spare."""
+    probs = [ms.square_inclusion_2d(N=N, side=0.3 + 0.5 * s / cells, a_incl=10.0) for s in range(cells)]
+    precision = hb.HOM_MIXED if prec == "mixed" else hb.HOM_FP64
+    out = solver.batched(probs, precision=precision, tol=1e-5)
+    if prec == "mixed":
+        assert launch(out) == want
+    try:
+        hb.binding.hom_set_batch_threads(solver.ctx, 256)
+        hb.binding.hom_set_batch_cluster(solver.ctx, 1, 0)
+        one = solver.batched(probs, precision=precision, tol=1e-5)
+    finally:
+        hb.binding.hom_set_batch_threads(solver.ctx, 0)
+        hb.binding.hom_set_batch_cluster(solver.ctx, 0, 0)
+    assert launch(one) == (256, 1) and (out["status"] == 0).all() and (one["status"] == 0).all()
+    for key in ("upper", "lower"):
+        for i in range(cells):
+            assert rel(out[key][i], one[key][i]) <= 1e-8, (key, i)
