@@ -103,11 +103,14 @@ __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t phase, long lo
 
 __device__ __forceinline__ float gelu(float x) { return 0.5f * x * (1.f + erff(x * 0.70710678118654752f)); }
 
-// PIPE: several chunks of K follow one another (a split of a long K): the next chunk's loads run
-// under this one's MMA, in registers (146 a thread). Else (K <= 64) a CTA walks row tiles with the
-// B tile staged once, eight CTAs an SM.
-template <bool PIPE>
-__global__ void __launch_bounds__(128, PIPE ? 3 : 8) k_gemm(GemmArgs g, int ksplit, float* partial) {
+// MULTI: several chunks of K, TA and TB as g.ta and g.tb. Bound by the chain of a chunk (loads, stores,
+// MMA), so by the loads in flight and, with many tiles, by the CTAs an SM: six, 80 registers. With the
+// next chunk's loads held in registers under the MMA (152, three CTAs) and divisions for every task's place
+// 2048 x 2048 x 512 took 91 us, 55 with one task's loads at a time in 48 registers and 54 so; 1024^3 89,
+// 77 and 52; 2048 x 1024 x 2048, A transposed, 237, 174 and 89 (calls with their 26 us of host work).
+// Else (K <= 64) a CTA walks row tiles with the B tile staged once, eight CTAs an SM.
+template <bool MULTI, bool TA = false, bool TB = false>
+__global__ void __launch_bounds__(128, MULTI ? 6 : 8) k_gemm(GemmArgs g, int ksplit, float* partial) {
   extern __shared__ __align__(1024) unsigned char smem[];
   unsigned char* sB = smem;                                 // [TBK/8][TBN/8][8][16 B]
   unsigned char* sA = smem + kStageOff;                     // [TBK/8][TBM/8][8][16 B]
@@ -119,6 +122,7 @@ __global__ void __launch_bounds__(128, PIPE ? 3 : 8) k_gemm(GemmArgs g, int kspl
   const float* A = g.A + (long long)bz * g.sA;
   const float* B = g.B + (long long)bz * g.sB;
   const int n0 = blockIdx.x * TBN, mtiles = (g.M + TBM - 1) / TBM;
+  const bool ta = MULTI ? TA : g.ta != 0, tb = MULTI ? TB : g.tb != 0;
   const int kchunk = ((g.K + ksplit - 1) / ksplit + TBK - 1) / TBK * TBK;
   const int kbeg = ks * kchunk;
   const int kend = min(g.K, kbeg + kchunk);
@@ -145,7 +149,7 @@ __global__ void __launch_bounds__(128, PIPE ? 3 : 8) k_gemm(GemmArgs g, int kspl
   const int cols = min(TBN, g.N - n0), cols8 = (cols + 7) & ~7;
   auto loadA = [&](float* v, int m0, int r, int kc, int k0) {
     const int gm = m0 + r, gk0 = k0 + kc * 8;
-    if (g.vecA && gm < g.M && gk0 + 8 <= kend) {   // two 16-byte loads along K
+    if (!ta && g.vecA && gm < g.M && gk0 + 8 <= kend) {   // two 16-byte loads along K
       const float4* p = reinterpret_cast<const float4*>(A + (long long)gm * g.lda + gk0);
       const float4 lo = __ldg(p), hi = __ldg(p + 1);
       v[0] = lo.x; v[1] = lo.y; v[2] = lo.z; v[3] = lo.w; v[4] = hi.x; v[5] = hi.y; v[6] = hi.z; v[7] = hi.w;
@@ -154,7 +158,7 @@ __global__ void __launch_bounds__(128, PIPE ? 3 : 8) k_gemm(GemmArgs g, int kspl
       for (int j = 0; j < 8; ++j) {
         const int gk = gk0 + j;
         v[j] = 0.f;
-        if (gm < g.M && gk < kend) v[j] = g.ta ? A[(long long)gk * g.lda + gm] : A[(long long)gm * g.lda + gk];
+        if (gm < g.M && gk < kend) v[j] = ta ? A[(long long)gk * g.lda + gm] : A[(long long)gm * g.lda + gk];
       }
     }
   };
@@ -164,14 +168,28 @@ __global__ void __launch_bounds__(128, PIPE ? 3 : 8) k_gemm(GemmArgs g, int kspl
     for (int j = 0; j < 8; ++j) {
       const int gk = k0 + kc * 8 + j;
       v[j] = 0.f;
-      if (gn < g.N && gk < kend) v[j] = g.tb ? B[(long long)gn * g.ldb + gk] : B[(long long)gk * g.ldb + gn];
+      if (gn < g.N && gk < kend) v[j] = tb ? B[(long long)gn * g.ldb + gk] : B[(long long)gk * g.ldb + gn];
     }
   };
   auto pack = [](const float* v) {
     return make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
   };
-  constexpr int NA = TBM * (TBK / 8) / 128, NB = TBN * (TBK / 8) / 128;
-  float va[PIPE ? NA : 1][8], vb[PIPE ? NB : 1][8];
+  auto storeA = [&](const float* v, int r, int kc) {
+    *reinterpret_cast<uint4*>(sA + ((kc * (TBM / 8) + (r >> 3)) * 8 + (r & 7)) * 16) = pack(v);
+  };
+  auto storeB = [&](const float* v, int n, int kc) {
+    *reinterpret_cast<uint4*>(sB + ((kc * (TBN / 8) + (n >> 3)) * 8 + (n & 7)) * 16) = pack(v);
+  };
+  auto stageA = [&](int m0, int r, int kc, int k0) {
+    float v[8];
+    loadA(v, m0, r, kc, k0);
+    storeA(v, r, kc);
+  };
+  auto stageB = [&](int n, int kc, int k0) {
+    float v[8];
+    loadB(v, n, kc, k0);
+    storeB(v, n, kc);
+  };
   // task c of a tile of `lines` rows or columns: its line and its K group, of kcn
   auto task = [](int c, bool along_k, int lines, int kcn, int& line, int& kc) {
     if (along_k) { line = c / kcn; kc = c - line * kcn; }
@@ -181,57 +199,71 @@ __global__ void __launch_bounds__(128, PIPE ? 3 : 8) k_gemm(GemmArgs g, int kspl
   for (int mt = blockIdx.y; mt < mtiles && ok; mt += gridDim.y) {
   const int m0 = mt * TBM;
   const int rows8 = (min(TBM, g.M - m0) + 7) & ~7;
-  if (PIPE && kbeg < kend) {
-#pragma unroll
-    for (int t = 0; t < NA; ++t)
-      if (tid + t * 128 < rows8 * (TBK / 8)) {
-        int r, kc;
-        task(tid + t * 128, !g.ta, rows8, TBK / 8, r, kc);
-        loadA(va[PIPE ? t : 0], m0, r, kc, kbeg);
-      }
-#pragma unroll
-    for (int t = 0; t < NB; ++t)
-      if (tid + t * 128 < cols8 * (TBK / 8)) {
-        int n, kc;
-        task(tid + t * 128, g.tb, cols8, TBK / 8, n, kc);
-        loadB(vb[PIPE ? t : 0], n, kc, kbeg);
-      }
-  }
   for (int k0 = kbeg; k0 < kend && ok; k0 += TBK) {
     // 8-element K groups up to the MMA's multiple of 16
-    const int kcn = PIPE ? TBK / 8 : (min(TBK, kend - k0) + 15) / 16 * 2;
-    // A tile, and B stored N x K (K-major)
-    if constexpr (PIPE) {
+    const int kcn = (min(TBK, kend - k0) + 15) / 16 * 2;
+    // A tile, and B stored N x K (K-major). Full tiles' tasks need no division to find; with several
+    // chunks, and where nothing ends inside the chunk, a thread has several tasks' loads in flight.
+    const bool whole = MULTI && k0 + TBK <= kend;
+    if (whole && m0 + TBM <= g.M && (TA || g.vecA)) {
+      const float* p = TA ? A + (long long)k0 * g.lda + m0 + tid : A + (long long)(m0 + (tid >> 3)) * g.lda + k0 + (tid & 7) * 8;
+      constexpr int U = TA ? 2 : 4;
+#pragma unroll 1
+      for (int t = 0; t < TBM / 16; t += U) {
+        float v[U][8];
 #pragma unroll
-      for (int t = 0; t < NA; ++t)
-        if (tid + t * 128 < rows8 * (TBK / 8)) {
-          int r, kc;
-          task(tid + t * 128, !g.ta, rows8, TBK / 8, r, kc);
-          *reinterpret_cast<uint4*>(sA + ((kc * (TBM / 8) + (r >> 3)) * 8 + (r & 7)) * 16) = pack(va[t]);
+        for (int u = 0; u < U; ++u) {
+          if (TA) {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) v[u][j] = p[(long long)((t + u) * 8 + j) * g.lda];
+          } else {
+            const float4* q = reinterpret_cast<const float4*>(p + (long long)(t + u) * 16 * g.lda);
+            const float4 lo = __ldg(q), hi = __ldg(q + 1);
+            v[u][0] = lo.x; v[u][1] = lo.y; v[u][2] = lo.z; v[u][3] = lo.w;
+            v[u][4] = hi.x; v[u][5] = hi.y; v[u][6] = hi.z; v[u][7] = hi.w;
+          }
         }
 #pragma unroll
-      for (int t = 0; t < NB; ++t)
-        if (tid + t * 128 < cols8 * (TBK / 8)) {
-          int n, kc;
-          task(tid + t * 128, g.tb, cols8, TBK / 8, n, kc);
-          *reinterpret_cast<uint4*>(sB + ((kc * (TBN / 8) + (n >> 3)) * 8 + (n & 7)) * 16) = pack(vb[t]);
-        }
+        for (int u = 0; u < U; ++u) storeA(v[u], TA ? tid : (tid >> 3) + 16 * (t + u), TA ? t + u : tid & 7);
+      }
+    } else if (rows8 == TBM && (MULTI || kcn == TBK / 8)) {
+      for (int c = tid; c < TBM * (TBK / 8); c += 128) {
+        const int r = ta ? c & (TBM - 1) : c >> 3, kc = ta ? c / TBM : c & 7;
+        if (kc < kcn) stageA(m0, r, kc, k0);
+      }
     } else {
       for (int c = tid; c < rows8 * kcn; c += 128) {
         int r, kc;
-        task(c, !g.ta, rows8, kcn, r, kc);
-        loadA(va[0], m0, r, kc, k0);
-        *reinterpret_cast<uint4*>(sA + ((kc * (TBM / 8) + (r >> 3)) * 8 + (r & 7)) * 16) = pack(va[0]);
+        task(c, !ta, rows8, kcn, r, kc);
+        stageA(m0, r, kc, k0);
       }
-      if (!haveB)
-        for (int c = tid; c < cols8 * kcn; c += 128) {
-          int n, kc;
-          task(c, g.tb, cols8, kcn, n, kc);
-          loadB(vb[0], n, kc, k0);
-          *reinterpret_cast<uint4*>(sB + ((kc * (TBN / 8) + (n >> 3)) * 8 + (n & 7)) * 16) = pack(vb[0]);
-        }
-      haveB = true;
     }
+    if (whole && n0 + TBN <= g.N) {
+      const int n = TB ? tid >> 3 : tid & (TBN - 1), kc = TB ? tid & 7 : tid / TBN;   // of the first task
+      const float* p = TB ? B + (long long)(n0 + n) * g.ldb + k0 + kc * 8 : B + (long long)(k0 + kc * 8) * g.ldb + n0 + n;
+#pragma unroll 1
+      for (int t = 0; t < TBN / 16; t += 2) {
+        float v[2][8];
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+#pragma unroll
+          for (int j = 0; j < 8; ++j) v[u][j] = p[TB ? (long long)(t + u) * 16 * g.ldb + j : (long long)((t + u) * 16 + j) * g.ldb];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) storeB(v[u], TB ? n + 16 * (t + u) : n, TB ? kc : kc + 2 * (t + u));
+      }
+    } else if (cols8 == TBN && (MULTI || (kcn == TBK / 8 && !haveB))) {
+      for (int c = tid; c < TBN * (TBK / 8); c += 128) {
+        const int n = tb ? c >> 3 : c & (TBN - 1), kc = tb ? c & 7 : c / TBN;
+        if (kc < kcn) stageB(n, kc, k0);
+      }
+    } else if (MULTI || !haveB) {
+      for (int c = tid; c < cols8 * kcn; c += 128) {
+        int n, kc;
+        task(c, tb, cols8, kcn, n, kc);
+        stageB(n, kc, k0);
+      }
+    }
+    haveB = true;
     // make the generic-proxy stores visible to the tensor core (async proxy)
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     __syncthreads();
@@ -251,22 +283,6 @@ __global__ void __launch_bounds__(128, PIPE ? 3 : 8) k_gemm(GemmArgs g, int kspl
       }
       asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar_a)
                    : "memory");
-    }
-    if (PIPE && k0 + TBK < kend) {
-#pragma unroll
-      for (int t = 0; t < NA; ++t)
-        if (tid + t * 128 < rows8 * (TBK / 8)) {
-          int r, kc;
-          task(tid + t * 128, !g.ta, rows8, TBK / 8, r, kc);
-          loadA(va[PIPE ? t : 0], m0, r, kc, k0 + TBK);
-        }
-#pragma unroll
-      for (int t = 0; t < NB; ++t)
-        if (tid + t * 128 < cols8 * (TBK / 8)) {
-          int n, kc;
-          task(tid + t * 128, g.tb, cols8, TBK / 8, n, kc);
-          loadB(vb[PIPE ? t : 0], n, kc, k0 + TBK);
-        }
     }
     ok = __syncthreads_and(mbar_wait(mbar_a, phase, g.spin) ? 1 : 0) != 0;   // one verdict for the CTA
     phase ^= 1u;
@@ -843,7 +859,11 @@ static cudaError_t launch_gemm(const GemmArgs& g, int gm, int gn, int ksplit, cu
     const int gy = (int)std::max<long long>(1, std::min<long long>(gm, 152 * 8 / others));
     k_gemm<false><<<dim3(gn, gy, g.batch * ksplit), 128, kGemmSmem, s>>>(g, ksplit, g_split_ws);
   } else {
-    k_gemm<true><<<dim3(gn, gm, g.batch * ksplit), 128, kGemmSmem, s>>>(g, ksplit, g_split_ws);
+    const dim3 grid(gn, gm, g.batch * ksplit);
+    if (g.ta && g.tb) k_gemm<true, true, true><<<grid, 128, kGemmSmem, s>>>(g, ksplit, g_split_ws);
+    else if (g.ta) k_gemm<true, true, false><<<grid, 128, kGemmSmem, s>>>(g, ksplit, g_split_ws);
+    else if (g.tb) k_gemm<true, false, true><<<grid, 128, kGemmSmem, s>>>(g, ksplit, g_split_ws);
+    else k_gemm<true, false, false><<<grid, 128, kGemmSmem, s>>>(g, ksplit, g_split_ws);
   }
   return cudaGetLastError();
 }

@@ -208,3 +208,24 @@ def test_long_rows_match_oracle(hb, solver, N, aniso):
     torch.cuda.synchronize()
     scale = max(np.abs(ref).max(), x.abs().max().item())
     assert np.abs(y.cpu().numpy() - ref).max() < 5e-6 * scale
+
+
+# full and partial tiles, K over one chunk, a ragged last chunk, strides that allow no vector loads
+@pytest.mark.parametrize("M,N,K,pad", [(128, 64, 64, 0), (128, 64, 128, 0), (256, 128, 192, 1), (200, 70, 100, 0), (129, 65, 65, 3),
+                                       (40, 24, 333, 0), (384, 192, 250, 4), (3, 2, 700, 0), (700, 64, 63, 2)])
+@pytest.mark.parametrize("ta,tb", [(0, 0), (0, 1), (1, 0), (1, 1)])
+def test_gemm_tiles(hb, solver, M, N, K, pad, ta, tb):
+    """The BF16 product against the same rounded operands in FP64: FP32 sums of K terms, at most
+    K 2^-23 of the sum of the terms' magnitudes."""
+    g = torch.Generator().manual_seed(M + N + K)
+    A = torch.randn((K, M) if ta else (M, K), generator=g)
+    B = torch.randn((N, K) if tb else (K, N), generator=g)
+    dA, dB = (torch.nn.functional.pad(t, (0, pad)).cuda() for t in (A, B))
+    C = torch.full((M, N + pad), 7.0, device="cuda")
+    hb.binding.hom_gemm_bf16(solver.ctx, M, N, K, dA.data_ptr(), dA.shape[1], ta, dB.data_ptr(), dB.shape[1], tb, C.data_ptr(),
+                             N + pad)
+    torch.cuda.synchronize()
+    a, b = (t.bfloat16().double() for t in (A.T if ta else A, B.T if tb else B))
+    err = (C[:, :N].cpu().double() - a @ b).abs()
+    assert (err <= K * 2.0 ** -23 * (a.abs() @ b.abs())).all()
+    assert (C[:, N:] == 7.0).all()
