@@ -803,11 +803,24 @@ __global__ void __launch_bounds__(kPassThreads) k_fft_batch(const cpx<T>* in, cp
 // shared-memory budget alone gives a 2D cell of N = 23 one to four CTAs a pass, each a chain of
 // transforms on one SM (its FP64 operator 45.8 -> 30.9 us, its bounds 3.31 -> 2.20 ms, the same
 // results). A grid that reaches this many CTAs keeps its larger chunks (3D N = 41: 528.6 us both).
+// rows > 0 (FP64 and float-float, whose passes are bound by a pipe of the SM): among the chunks from
+// there up to the budget's, the one that leaves the fullest SM the fewest pencils (two rows each
+// in a row pass of `rows` rows a plane, else rows = 2): with the cut alone a third CTA on two SMs
+// (306 of them) took the FP64 operator at N = 23 in 3D from 124 to 129 us, and two rounds of two
+// pencils for one of three at N = 203 in 2D from 113 to 118; so 110 and 112. FP32 is
+// bound by latency there: more CTAs an SM are faster however they divide (N = 203: 26 us, 30 so).
 constexpr long long kSpreadCtas = 304;
-inline long long spread_chunk(long long chunk, long long n, long long others) {
-  if (others < 1 || chunk < 2 || ((n + chunk - 1) / chunk) * others >= kSpreadCtas) return chunk;
+inline long long spread_chunk(long long chunk, long long n, long long others, int rows = 0) {
+  auto ctas = [=](long long c) { return ((n + c - 1) / c) * others; };
+  if (others < 1 || chunk < 2 || ctas(chunk) >= kSpreadCtas) return chunk;
   const long long want = std::min(n, (kSpreadCtas + others - 1) / others);
-  return (n + want - 1) / want;
+  long long best = (n + want - 1) / want;
+  if (rows > 0) {
+    auto fullest = [&](long long c) { return (ctas(c) + 151) / 152 * ((c * rows + 1) / 2); };
+    for (long long c = best + 1; c <= chunk; ++c)
+      if (fullest(c) < fullest(best)) best = c;
+  }
+  return best;
 }
 
 // Threads of a pass CTA with G pencils of length M: one per smallest (radix 3) butterfly, or the
@@ -866,7 +879,7 @@ template <typename T> int pencil_xc_fit(int M, int X, int C) {
 }
 
 template <typename T> int pencil_xc(int M, int X, int C, long long slabs) {
-  return (int)spread_chunk(pencil_xc_fit<T>(M, X, C), X, slabs);
+  return (int)spread_chunk(pencil_xc_fit<T>(M, X, C), X, slabs, sizeof(cpx<T>) == 16 ? 2 : 0);
 }
 
 template <typename T> int xpass_yb_fit(int M, int rpp, int planes) {
@@ -900,7 +913,7 @@ template <typename T> int xpass_yb_fit(int M, int rpp, int planes) {
 }
 
 template <typename T> int xpass_yb(int M, int rpp, int planes, int gy) {
-  return (int)spread_chunk(xpass_yb_fit<T>(M, rpp, planes), planes, gy);
+  return (int)spread_chunk(xpass_yb_fit<T>(M, rpp, planes), planes, gy, sizeof(cpx<T>) == 16 ? rpp : 0);
 }
 
 template <typename T, int MT> cudaError_t launch_pencil_m(PencilArgs a, cudaStream_t s) {
