@@ -973,7 +973,14 @@ __device__ __forceinline__ void dft3_mid_in0(cpx<T>* v, int dir) {   // v[1] == 
   const cpx<T> a = v[0], c = v[2];
   const cpx<T> t2 = axpy<T>(-h, c, a);
   v[0] = add<T>(a, c);
-  dft3_sine<T>(t2, mk<T>(-c.x, -c.y), dir, &v[1], &v[2]);
+  if constexpr (sine_fma<T>::value) {
+    dft3_sine<T>(t2, mk<T>(-c.x, -c.y), dir, &v[1], &v[2]);
+  } else {   // the order of a float-float product's factors is part of its rounding
+    const T s3 = T(0.86602540378443864676372317075294);
+    const cpx<T> it3 = rot<T>(mk<T>(-s3 * c.x, -s3 * c.y), dir > 0 ? 1 : -1);
+    v[1] = add<T>(t2, it3);
+    v[2] = sub<T>(t2, it3);
+  }
 }
 template <typename T>
 __device__ __forceinline__ void dft3_skip_out1(cpx<T>* v, int dir) {   // v[1] left undefined
