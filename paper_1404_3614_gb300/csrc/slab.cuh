@@ -23,10 +23,11 @@
 
 namespace homb {
 
-// 16 warps at 128 registers a thread (what the kernel takes), and, at a caller's request for more,
-// 20 warps at 96 in a compilation of their own (R < 15: 20 warps' scratch at 225 exceeds the
-// shared memory)
-constexpr int kSlabMaxThreads = 512, kSlabWideThreads = 640;
+// 15 warps, and, where a caller asks for more, a compilation for 20 (at 225 for 16: 20 warps' scratch
+// exceeds the shared memory). One compilation for 16 warps costs the 15 of the automatic choice at
+// 225 0.7 % (operator 382.8 -> 385.5 us).
+constexpr int kSlabMaxThreads = 480;
+constexpr int slab_wide_threads(int R) { return R < 15 ? 640 : 512; }
 
 // Layout of the slab in shared memory: columns kx = l + R m and l + R (m + 1), m even, side by side
 // (a column pair: one lane group's two pencils in the y passes, and two of a lane's values
@@ -554,9 +555,7 @@ template <int R, bool ZB, int NT> cudaError_t launch_slab_nt(const SlabArgs& a, 
 }
 
 template <int R, bool ZB> cudaError_t launch_slab_rz(const SlabArgs& a, int warps, cudaStream_t s) {
-  if constexpr (R < 15) {
-    if (warps * 32 > kSlabMaxThreads) return launch_slab_nt<R, ZB, kSlabWideThreads>(a, warps, s);
-  }
+  if (warps * 32 > kSlabMaxThreads) return launch_slab_nt<R, ZB, slab_wide_threads(R)>(a, warps, s);
   return launch_slab_nt<R, ZB, kSlabMaxThreads>(a, warps, s);
 }
 
@@ -608,7 +607,7 @@ template <typename T> int slab_warps_asked(int M, int Ny, int Nh, int asked) {
   const int warps = slab_warps<T>(M, Ny, Nh);
   if (warps == 0 || asked <= 0) return warps;
   const int r = M == 225 ? 15 : (M == 81 ? 9 : (M == 25 ? 5 : 3));
-  const bool fits = asked * 32 <= (r < 15 ? kSlabWideThreads : kSlabMaxThreads) &&
+  const bool fits = asked * 32 <= slab_wide_threads(r) &&
                     slab_smem_bytes(r, slab_band_free(M, Ny, Nh), Ny, Nh, asked) <= 227 * 1024;
   return fits ? asked : warps;
 }
