@@ -172,13 +172,8 @@ assert _INCLUSION.size == C.sizeof(hom_inclusion) and _PROBLEM.size == C.sizeof(
 
 def _vector(v, n, fill):
     """v (an array of at most three entries, or one value for n of them) as three floats."""
-    if type(v) is np.ndarray and v.ndim == 1:
-        v = v.tolist()
-        if len(v) == 1 and n > 1:
-            v = v * n
-        elif len(v) != n:
-            raise ValueError(f"expected {n} values, got {len(v)}")
-        return v + [fill] * (3 - n)
+    if type(v) is np.ndarray and v.shape == (n,) and n <= 3 and v.dtype.kind in "fiu":
+        return v.tolist() + [fill] * (3 - n)
     out = np.full(3, fill)
     out[:n] = v
     return out.tolist()
@@ -186,7 +181,7 @@ def _vector(v, n, fill):
 
 def _tensor(A, d):
     """A (d x d, or one value for every entry) row-major in a 3 x 3 block."""
-    if type(A) is np.ndarray and A.shape == (d, d):
+    if type(A) is np.ndarray and A.shape == (d, d) and 2 <= d <= 3 and A.dtype.kind in "fiu":
         r = A.tolist()
         return r[0] + r[1] + r[2] if d == 3 else [*r[0], 0.0, *r[1], 0.0, 0.0, 0.0, 0.0]
     return _mat3(A, d).tolist()
@@ -212,6 +207,8 @@ def problem_struct(problem):
         img = np.ascontiguousarray(np.asarray(bm, dtype=np.float64).T)
         img_at = img.ctypes.data
         P[:d] = list(bm.shape)
+        if len(P) != 3:
+            raise ValueError(f"a {len(bm.shape)}-dimensional image in {d} dimensions")
         keep.append(img)
     p = hom_problem.from_buffer(bytearray(_PROBLEM.pack(
         d, *map(int, N), *([1] * (3 - d)), *_vector(problem.Y, d, 1.0), *_tensor(problem.A0, d), n, 0, C.addressof(owner),

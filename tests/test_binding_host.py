@@ -68,3 +68,36 @@ def test_one_value_fills_every_axis(bd):
     assert list(p.N) == [7, 7, 1] and list(p.Y) == [1.0, 1.0, 1.0] and p.closed == 1
     assert list(p.A0)[:5] == [1.5, 1.5, 0.0, 1.5, 1.5]
     assert list(p.bitmap_n) == [2, 3, 1] and p.bitmap[:6] == [0.0, 3.0, 1.0, 4.0, 2.0, 5.0]
+
+
+class Description:
+    """A problem of one size in every direction; members replaced by keyword."""
+    def __init__(self, d, **kw):
+        self.d, self.N, self.Y, self.A0, self.inclusions = d, np.full(d, 5), np.ones(d), np.eye(d), []
+        self.__dict__.update(kw)
+
+
+@pytest.mark.parametrize("d", [0, 1])
+def test_other_dimensions_reach_the_library(bd, d):
+    """The library refuses them by its status; the binding only passes them on."""
+    p, keep = bd.problem_struct(Description(d))
+    assert p.d == d and list(p.N) == [5] * d + [1] * (3 - d) and list(p.A0) == [1.0 * (d == 1)] + [0.0] * 8
+
+
+@pytest.mark.parametrize("kw", [dict(d=4), dict(d=2, N=np.full(3, 5)), dict(d=3, Y=np.ones(2)), dict(d=2, A0=np.eye(3)),
+                                dict(d=2, inclusions=[ms.Inclusion("box", np.zeros(2), np.ones(4), np.eye(2))]),
+                                dict(d=2, inclusions=[ms.Inclusion("box", np.zeros(3), np.ones(2), np.eye(2))]),
+                                dict(d=2, bitmap=np.ones(3)), dict(d=2, bitmap=np.ones((3, 4, 5)))],
+                         ids=lambda kw: ",".join(kw))
+def test_shapes_that_do_not_fit_are_value_errors(bd, kw):
+    with pytest.raises(ValueError):
+        bd.problem_struct(Description(**kw))
+
+
+def test_other_number_types(bd):
+    """Complex values keep their real part (numpy warns), as every array that is assigned to floats."""
+    with pytest.warns(np.exceptions.ComplexWarning):
+        p, keep = bd.problem_struct(Description(2, Y=np.array([1 + 1j, 2.0]), A0=np.eye(2) * (3 + 0j)))
+    assert list(p.Y) == [1.0, 2.0, 1.0] and list(p.A0)[:5] == [3.0, 0.0, 0.0, 0.0, 3.0]
+    p, keep = bd.problem_struct(Description(2, Y=np.array([2.0]), N=np.array([7])))
+    assert list(p.Y) == [2.0, 2.0, 1.0] and list(p.N) == [7, 7, 1]
