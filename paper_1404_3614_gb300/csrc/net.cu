@@ -549,7 +549,7 @@ __global__ void __launch_bounds__(256) k_gemm_tn(GemmArgs g, int ksplit, float* 
 // of which the second adds to the first's result):
 //   kPairs     C0 = A0 B0 + s01 A1 B1, C1 = t0 A0 B1 + t1 A1 B0   (complex products)
 //   kTwoLeft   C0 = A0 B0, C1 = A1 B0                             (real data onto two bases)
-//   kSum       C0 = (beta C0 + A0 B0) + A1 B1                     (two bases back to real data)
+//   kSum       C0 = (C0 +) A0 B0 + A1 B1, added in this order     (two bases back to real data)
 // Against a launch per product, each with one 128 x 64 tile per batch item: these products
 // have 8 to 63 rows and 24 or 32 columns an item, and what they cost is the tiles' set-up and the
 // loads of their operands. Here a CTA walks tiles, keeps a shared basis staged, fills a
@@ -563,7 +563,8 @@ struct ProdArgs {
   int M, N, K, lda, ldb, ldc, ta, tb;
   long long sA, sB, sC;
   int batch;
-  float s01, t0, t1, beta;
+  float s01, t0, t1;
+  int add;              // kSum: to what is in C0
   int per;              // batch items in a tile's columns (N <= 64 / per), or 0: one item, N in tiles of 64
   int mt, nt;           // tiles along M; along N (per = 0) or groups of items
   uint32_t items;
@@ -766,7 +767,7 @@ __global__ void __launch_bounds__(128, MODE == kPairs ? 2 : 4) k_prod(ProdArgs g
             if (g.vecC) {   // N, the strides and the base are multiples of four floats
               float4 w = make_float4(o[j4], o[j4 + 1], o[j4 + 2], o[j4 + 3]);
               if (MODE == kSum) {
-                if (g.beta != 0.f) {
+                if (g.add) {
                   const float4 c4 = *reinterpret_cast<const float4*>(d);
                   w.x += c4.x; w.y += c4.y; w.z += c4.z; w.w += c4.w;
                 }
@@ -780,7 +781,7 @@ __global__ void __launch_bounds__(128, MODE == kPairs ? 2 : 4) k_prod(ProdArgs g
                             (g.per > 0 ? n + e - je * g.N : n0 + n + e);
                 float w = o[j4 + e];
                 if (MODE == kSum) {
-                  if (g.beta != 0.f) w += *de;
+                  if (g.add) w += *de;
                   w += p[1][j4 + e];
                 }
                 *de = w;
@@ -846,7 +847,7 @@ static cudaError_t launch_gemm(const GemmArgs& g, int gm, int gn, int ksplit, cu
   // long splits of A^T B whose rows can be copied in 16-byte pieces
   if (ksplit > 1 && g.batch == 1 && g.ta && !g.tb && g.M % 4 == 0 && g.N % 4 == 0 && g.lda % 4 == 0 && g.ldb % 4 == 0 &&
       ((reinterpret_cast<uintptr_t>(g.A) | reinterpret_cast<uintptr_t>(g.B)) & 15) == 0) {
-    // 200 KB at most (128 rows, 64 columns): one CTA an SM then, and tensor memory for its 64 columns
+    // 216 KB at most (128 rows, 64 columns): one CTA an SM then, and tensor memory for its 64 columns
     static std::atomic<int> cache[kAttrDevices] = {};
     const size_t smem = tn_smem(std::min(g.M, TBM), std::min(g.N, TBN));
     const cudaError_t e = smem_attr(k_gemm_tn, smem, cache);
@@ -1403,7 +1404,7 @@ cudaError_t net_backward(const NetConfig& c, const float* prm, const float* base
     // (1') dv += Fr^T dX1r + Fi^T dX1i, per (b, (z,) y): [N x K] x [K x W]
     ProdArgs dv = prod(bs.Fr, bs.Fi, w.dx1r, w.dx1i, w.dv, nullptr, N, W, K, N, W, W, 1, 0, 0, (long long)K * W,
                        (long long)N * W, BN);
-    dv.beta = 1.f;
+    dv.add = 1;
     NCK(run_prod<kSum>(dv, s));
   }
   // lift
