@@ -584,7 +584,8 @@ template <typename T> int slab_warps(int M, int Ny, int Nh) {
   // leave 32 mod R lanes of every warp issuing FP64 work on zeros
   if (R == 0 || sizeof(T) == 8) return 0;
   // the warps with the least idle lane groups over the rounds (two rounds of column pairs, weight 1
-  // each, and of row groups, weight 2.2), more warps where that ties: 225: 15, 81: 7, 25: 2, 9: 1
+  // each, and of row groups, weight 2.2), more warps where that ties: zero-padded 225: 15, 81: 7, 25: 1,
+  // 9: 1; as long as the data 81: 9, 25: 2, 9: 1
   const bool zb = slab_band_free(M, Ny, Nh);
   const int PW = 32 / R, nc = slab_pairs(R, zb), nquad = (M + 3) / 4;
   int best = 0;

@@ -233,3 +233,9 @@ def test_asked_warps_are_taken_where_they_fit(exe, M, N):
     assert auto > 0
     for asked in (4, 8, 12, 16, 20):
         assert warps_of(exe, M, N, asked) == (auto if (M, asked) == (225, 20) else asked)
+
+
+@pytest.mark.parametrize("M,N,warps", [(225, 113, 15), (81, 41, 7), (25, 13, 1), (9, 5, 1), (81, 81, 9), (25, 25, 2), (9, 9, 1)])
+def test_automatic_warps(exe, M, N, warps):
+    """The counts that the rule's comment names."""
+    assert warps_of(exe, M, N, 0) == warps
