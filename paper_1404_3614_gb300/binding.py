@@ -172,8 +172,17 @@ assert _INCLUSION.size == C.sizeof(hom_inclusion) and _PROBLEM.size == C.sizeof(
 
 def _vector(v, n, fill):
     """v (an array of at most three entries, or one value for n of them) as three floats."""
-    if type(v) is np.ndarray and v.shape == (n,) and n <= 3 and v.dtype.kind in "fiu":
-        return v.tolist() + [fill] * (3 - n)
+    if type(v) is np.ndarray and v.ndim == 1:
+        v = v.tolist()
+        if len(v) == 1 and n > 1:
+            v = v * n
+        elif len(v) != n:
+            raise ValueError(f"expected {n} values, got {len(v)}")
+        return v + [fill] * (3 - n)
+    return _vector_any(v, n, fill)
+
+
+def _vector_any(v, n, fill):
     out = np.full(3, fill)
     out[:n] = v
     return out.tolist()
@@ -181,7 +190,7 @@ def _vector(v, n, fill):
 
 def _tensor(A, d):
     """A (d x d, or one value for every entry) row-major in a 3 x 3 block."""
-    if type(A) is np.ndarray and A.shape == (d, d) and 2 <= d <= 3 and A.dtype.kind in "fiu":
+    if type(A) is np.ndarray and A.shape == (d, d):
         r = A.tolist()
         return r[0] + r[1] + r[2] if d == 3 else [*r[0], 0.0, *r[1], 0.0, 0.0, 0.0, 0.0]
     return _mat3(A, d).tolist()
@@ -189,17 +198,26 @@ def _tensor(A, d):
 
 def problem_struct(problem):
     """hom_problem from a microstructures.Problem. Returns (struct, keepalive)."""
+    try:
+        return _pack(problem, _vector, _tensor)
+    except (struct.error, IndexError, ValueError):
+        pass
+    # other dimensions and number types: as numpy assigns them, its errors where it refuses
+    return _pack(problem, _vector_any, lambda A, d: _mat3(A, d).tolist())
+
+
+def _pack(problem, vector, tensor):
     d = int(problem.d)
     n = len(problem.inclusions)
     arr = bytearray(_INCLUSION.size * max(n, 1))
     at = 0
     for inc in problem.inclusions:
-        _INCLUSION.pack_into(arr, at, HOM_BOX if inc.shape == "box" else HOM_BALL, 0, *_vector(inc.center, d, 0.0),
-                             *_vector(inc.size, len(inc.size), 0.0), *_tensor(inc.A, d))
+        _INCLUSION.pack_into(arr, at, HOM_BOX if inc.shape == "box" else HOM_BALL, 0, *vector(inc.center, d, 0.0),
+                             *vector(inc.size, len(inc.size), 0.0), *tensor(inc.A, d))
         at += _INCLUSION.size
     owner = C.c_char.from_buffer(arr)
     keep = [arr, owner]
-    N = problem.N.tolist() if type(problem.N) is np.ndarray and problem.N.shape == (d,) else _vector(problem.N, d, 1.0)[:d]
+    N = problem.N.tolist() if type(problem.N) is np.ndarray and problem.N.shape == (d,) else vector(problem.N, d, 1.0)[:d]
     bm = getattr(problem, "bitmap", None)
     img_at, P = 0, [1, 1, 1]
     if bm is not None:
@@ -211,7 +229,7 @@ def problem_struct(problem):
             raise ValueError(f"a {len(bm.shape)}-dimensional image in {d} dimensions")
         keep.append(img)
     p = hom_problem.from_buffer(bytearray(_PROBLEM.pack(
-        d, *map(int, N), *([1] * (3 - d)), *_vector(problem.Y, d, 1.0), *_tensor(problem.A0, d), n, 0, C.addressof(owner),
+        d, *map(int, N), *([1] * (3 - d)), *vector(problem.Y, d, 1.0), *tensor(problem.A0, d), n, 0, C.addressof(owner),
         img_at, *P, 1 if getattr(problem, "closed", False) else 0, 1 if getattr(problem, "smooth", False) else 0)))
     return p, keep
 

@@ -807,16 +807,17 @@ __global__ void __launch_bounds__(kPassThreads) k_fft_batch(const cpx<T>* in, cp
 // there up to the budget's, the one that leaves the fullest SM the fewest pencils (two rows each
 // in a row pass of `rows` rows a plane, else rows = 2): with the cut alone a third CTA on two SMs
 // (306 of them) took the FP64 operator at N = 23 in 3D from 124 to 129 us, and two rounds of two
-// pencils for one of three at N = 203 in 2D from 113 to 118; so 110 and 112. FP32 is
-// bound by latency there: more CTAs an SM are faster however they divide (N = 203: 26 us, 30 so).
+// pencils for one of three at N = 203 in 2D from 113 to 118; so 110 and 112. Short of 1200 points on
+// that SM, and in FP32, the passes are bound by latency, and more CTAs an SM are faster however they
+// divide (FP32, N = 203: 26 us, 30 so; float-float, N = 113 in 2D, 900 points: 54.7 and 56.7).
 constexpr long long kSpreadCtas = 304;
-inline long long spread_chunk(long long chunk, long long n, long long others, int rows = 0) {
+inline long long spread_chunk(long long chunk, long long n, long long others, int rows = 0, int M = 0) {
   auto ctas = [=](long long c) { return ((n + c - 1) / c) * others; };
   if (others < 1 || chunk < 2 || ctas(chunk) >= kSpreadCtas) return chunk;
   const long long want = std::min(n, (kSpreadCtas + others - 1) / others);
   long long best = (n + want - 1) / want;
-  if (rows > 0) {
-    auto fullest = [&](long long c) { return (ctas(c) + 151) / 152 * ((c * rows + 1) / 2); };
+  auto fullest = [&](long long c) { return (ctas(c) + 151) / 152 * ((c * rows + 1) / 2); };
+  if (fullest(best) * M >= 1200) {
     for (long long c = best + 1; c <= chunk; ++c)
       if (fullest(c) < fullest(best)) best = c;
   }
@@ -879,7 +880,7 @@ template <typename T> int pencil_xc_fit(int M, int X, int C) {
 }
 
 template <typename T> int pencil_xc(int M, int X, int C, long long slabs) {
-  return (int)spread_chunk(pencil_xc_fit<T>(M, X, C), X, slabs, sizeof(cpx<T>) == 16 ? 2 : 0);
+  return (int)spread_chunk(pencil_xc_fit<T>(M, X, C), X, slabs, sizeof(cpx<T>) == 16 ? 2 : 0, M);
 }
 
 template <typename T> int xpass_yb_fit(int M, int rpp, int planes) {
@@ -913,7 +914,7 @@ template <typename T> int xpass_yb_fit(int M, int rpp, int planes) {
 }
 
 template <typename T> int xpass_yb(int M, int rpp, int planes, int gy) {
-  return (int)spread_chunk(xpass_yb_fit<T>(M, rpp, planes), planes, gy, sizeof(cpx<T>) == 16 ? rpp : 0);
+  return (int)spread_chunk(xpass_yb_fit<T>(M, rpp, planes), planes, gy, sizeof(cpx<T>) == 16 ? rpp : 0, M);
 }
 
 template <typename T, int MT> cudaError_t launch_pencil_m(PencilArgs a, cudaStream_t s) {

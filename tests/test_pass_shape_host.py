@@ -23,7 +23,7 @@ int main(int argc, char**) {
       for (int others : {1, 2, 3, 4, 9, 40, 151, 400})
         for (int n : {1, 2, 3, 12, 57, 102, 276, 405, 2025, 6561})
           for (int chunk : {1, 2, 3, 7, 22, 33, 64})
-            std::printf("%%d %%d %%d %%d %%lld\n", rows, others, n, chunk, spread_chunk(chunk, n, others, rows));
+            std::printf("%%d %%d %%d %%d %%lld\n", rows, others, n, chunk, spread_chunk(chunk, n, others, rows, 1200));
     return 0;
   }
   for (int rpp = 2; rpp <= 3; ++rpp)
