@@ -195,14 +195,17 @@ inline void make_plan(int M, FftPlan& p, bool big = true) {
 // FMA for each part: a packed product would be rounded by itself (the scalar one is contracted into
 // the sums) and takes two operations more in fpair. Against 64 bits: FP32 operator at N = 203 in 2D 1.66e-7
 // -> 1.61e-7 (1.60e-7 in scalars), N = 113 in 3D 1.64e-7 -> 1.62e-7 (1.62e-7), the same time.
+// F = false: the packed product, in the runtime plans, whose other radices round less than before as it
+// is (ragged 41 x 33 x 53 cell 1.57e-7 in scalars, 1.51e-7 so) and which the FMAs make slower
+// at some lengths (N = 255 in 2D 95 -> 97 us, N = 17 21.0 -> 22.5).
 template <typename T> struct sine_fma { static constexpr bool value = is_fpair<T>::value; };
 #if defined(__CUDA_ARCH__) && !defined(HOMB_SCALAR_COMPLEX)
 template <> struct sine_fma<float> { static constexpr bool value = true; };
 #endif
-template <typename T>
+template <typename T, bool F = sine_fma<T>::value>
 __device__ __forceinline__ void dft3_sine(cpx<T> t, cpx<T> d, int dir, cpx<T>* v1, cpx<T>* v2) {
   const T s3 = T(0.86602540378443864676372317075294);
-  if constexpr (sine_fma<T>::value) {
+  if constexpr (F) {
     const T p = dir > 0 ? s3 : -s3, n = dir > 0 ? -s3 : s3;
     *v1 = mk<T>(fma(n, d.y, t.x), fma(p, d.x, t.y));
     *v2 = mk<T>(fma(p, d.y, t.x), fma(n, d.x, t.y));
@@ -212,12 +215,12 @@ __device__ __forceinline__ void dft3_sine(cpx<T> t, cpx<T> d, int dir, cpx<T>* v
     *v2 = sub<T>(t, it3);
   }
 }
-template <typename T> __device__ __forceinline__ void dft3(cpx<T>* v, int dir) {
+template <typename T, bool F = sine_fma<T>::value> __device__ __forceinline__ void dft3(cpx<T>* v, int dir) {
   const T h = T(0.5);
   const cpx<T> t1 = add<T>(v[1], v[2]), d = sub<T>(v[1], v[2]);
   const cpx<T> t2 = axpy<T>(-h, t1, v[0]);
   v[0] = add<T>(v[0], t1);
-  dft3_sine<T>(t2, d, dir, &v[1], &v[2]);   // forward: V1 = t2 - i s3 d, V2 = t2 + i s3 d
+  dft3_sine<T, F>(t2, d, dir, &v[1], &v[2]);   // forward: V1 = t2 - i s3 d, V2 = t2 + i s3 d
 }
 
 template <typename T> __device__ __forceinline__ void dft5(cpx<T>* v, int dir) {
@@ -336,7 +339,7 @@ __device__ __forceinline__ void dft_ct(cpx<T>* v, int dir) {
 // Length 15 by the prime-factor (Good-Thomas) map, 15 = 3 * 5 with coprime factors:
 // input n = (5 n1 + 3 n2) mod 15, output k = (10 k1 + 6 k2) mod 15, so that
 // w_15^(n k) = w_3^(n1 k1) w_5^(n2 k2) and no twiddle multiplications are needed.
-template <typename T>
+template <typename T, bool F = sine_fma<T>::value>
 __device__ __forceinline__ void dft15_pfa(cpx<T>* v, int dir) {
   cpx<T> t[15];
 #pragma unroll
@@ -344,7 +347,7 @@ __device__ __forceinline__ void dft15_pfa(cpx<T>* v, int dir) {
     cpx<T> a[3];
 #pragma unroll
     for (int n1 = 0; n1 < 3; ++n1) a[n1] = v[(5 * n1 + 3 * n2) % 15];
-    dft3<T>(a, dir);
+    dft3<T, F>(a, dir);
 #pragma unroll
     for (int k1 = 0; k1 < 3; ++k1) t[n2 * 3 + k1] = a[k1];
   }
@@ -497,7 +500,7 @@ __device__ __forceinline__ void dft15_zin(cpx<T>* v, int dir) {
 
 // Length-15 DFT (prime-factor map) computing only the outputs outside the zero band (0..3,
 // 11..14); the band's outputs are left undefined.
-template <typename T>
+template <typename T, bool F = sine_fma<T>::value>
 __device__ __forceinline__ void dft15_zout(cpx<T>* v, int dir) {
   cpx<T> t[15];
 #pragma unroll
@@ -505,7 +508,7 @@ __device__ __forceinline__ void dft15_zout(cpx<T>* v, int dir) {
     cpx<T> a[3];
 #pragma unroll
     for (int n1 = 0; n1 < 3; ++n1) a[n1] = v[(5 * n1 + 3 * n2) % 15];
-    dft3<T>(a, dir);
+    dft3<T, F>(a, dir);
 #pragma unroll
     for (int k1 = 0; k1 < 3; ++k1) t[n2 * 3 + k1] = a[k1];
   }
@@ -585,16 +588,16 @@ __device__ __forceinline__ void dft_odd(cpx<T>* v) {
 }
 
 // Radix 9 = 3 x 3 with its middle inputs 3..5 zero (ZI) or its middle outputs 3..5 not needed (ZO)
-template <typename T> __device__ __forceinline__ void dft3_mid_in0(cpx<T>* v, int dir);
-template <typename T> __device__ __forceinline__ void dft3_skip_out1(cpx<T>* v, int dir);
+template <typename T, bool F = sine_fma<T>::value> __device__ __forceinline__ void dft3_mid_in0(cpx<T>* v, int dir);
+template <typename T, bool F = sine_fma<T>::value> __device__ __forceinline__ void dft3_skip_out1(cpx<T>* v, int dir);
 template <typename T, int DIR, bool ZI, bool ZO>
 __device__ __forceinline__ void dft9_band(cpx<T>* v) {
   cpx<T> t[9];
 #pragma unroll
   for (int n2 = 0; n2 < 3; ++n2) {
     cpx<T> a[3] = {v[n2], v[3 + n2], v[6 + n2]};
-    if (ZI) dft3_mid_in0<T>(a, DIR);
-    else dft3<T>(a, DIR);
+    if (ZI) dft3_mid_in0<T, false>(a, DIR);
+    else dft3<T, false>(a, DIR);
 #pragma unroll
     for (int k1 = 0; k1 < 3; ++k1) {
       if (n2 * k1 == 0) {
@@ -608,8 +611,8 @@ __device__ __forceinline__ void dft9_band(cpx<T>* v) {
 #pragma unroll
   for (int k1 = 0; k1 < 3; ++k1) {
     cpx<T> b[3] = {t[k1], t[3 + k1], t[6 + k1]};
-    if (ZO) dft3_skip_out1<T>(b, DIR);
-    else dft3<T>(b, DIR);
+    if (ZO) dft3_skip_out1<T, false>(b, DIR);
+    else dft3<T, false>(b, DIR);
     v[k1] = b[0];
     if (!ZO) v[3 + k1] = b[1];
     v[6 + k1] = b[2];
@@ -651,13 +654,13 @@ __device__ __forceinline__ void dft_pow2(cpx<T>* v) {
 template <typename T, int R, int DIR, bool ZI, bool ZO>
 __device__ __forceinline__ void dft_radix(cpx<T>* v) {
   if constexpr (R % 2 == 0) dft_pow2<T, R, DIR>(v);
-  else if constexpr (R == 3 && ZI) dft3_mid_in0<T>(v, DIR);
-  else if constexpr (R == 3 && ZO) dft3_skip_out1<T>(v, DIR);
-  else if constexpr (R == 3) dft3<T>(v, DIR);
+  else if constexpr (R == 3 && ZI) dft3_mid_in0<T, false>(v, DIR);
+  else if constexpr (R == 3 && ZO) dft3_skip_out1<T, false>(v, DIR);
+  else if constexpr (R == 3) dft3<T, false>(v, DIR);
   else if constexpr (R == 9) dft9_band<T, DIR, ZI, ZO>(v);
   else if constexpr (R == 15 && ZI) dft15_zin<T>(v, DIR);
-  else if constexpr (R == 15 && ZO) dft15_zout<T>(v, DIR);
-  else if constexpr (R == 15) dft15_pfa<T>(v, DIR);
+  else if constexpr (R == 15 && ZO) dft15_zout<T, false>(v, DIR);
+  else if constexpr (R == 15) dft15_pfa<T, false>(v, DIR);
   else if constexpr (R == 5 && !ZI && !ZO) dft5<T>(v, DIR);
   else dft_odd<T, R, DIR, ZI, ZO>(v);
 }
@@ -967,14 +970,14 @@ __device__ __forceinline__ void cbfly(const cpx<T>* __restrict__ src, cpx<T>* __
 
 // Radix-3 butterflies of a first stage whose middle inputs are all zero (a zero-padded
 // spectrum), and of a last stage whose middle outputs are not needed (a truncated one).
-template <typename T>
+template <typename T, bool F>
 __device__ __forceinline__ void dft3_mid_in0(cpx<T>* v, int dir) {   // v[1] == 0
   const T h = T(0.5);
   const cpx<T> a = v[0], c = v[2];
   const cpx<T> t2 = axpy<T>(-h, c, a);
   v[0] = add<T>(a, c);
-  if constexpr (sine_fma<T>::value) {
-    dft3_sine<T>(t2, mk<T>(-c.x, -c.y), dir, &v[1], &v[2]);
+  if constexpr (F) {
+    dft3_sine<T, F>(t2, mk<T>(-c.x, -c.y), dir, &v[1], &v[2]);
   } else {   // the order of a float-float product's factors is part of its rounding
     const T s3 = T(0.86602540378443864676372317075294);
     const cpx<T> it3 = rot<T>(mk<T>(-s3 * c.x, -s3 * c.y), dir > 0 ? 1 : -1);
@@ -982,13 +985,13 @@ __device__ __forceinline__ void dft3_mid_in0(cpx<T>* v, int dir) {   // v[1] == 
     v[2] = sub<T>(t2, it3);
   }
 }
-template <typename T>
+template <typename T, bool F>
 __device__ __forceinline__ void dft3_skip_out1(cpx<T>* v, int dir) {   // v[1] left undefined
   const T h = T(0.5);
   const cpx<T> t1 = add<T>(v[1], v[2]), d = sub<T>(v[1], v[2]);
   const cpx<T> t2 = axpy<T>(-h, t1, v[0]);
   v[0] = add<T>(v[0], t1);
-  dft3_sine<T>(t2, d, dir, &v[1], &v[2]);
+  dft3_sine<T, F>(t2, d, dir, &v[1], &v[2]);
 }
 
 // prune bit 1: the first stage (radix 3, stride nb = M/3) reads only inputs j and j + 2 nb
