@@ -225,10 +225,11 @@ __device__ __forceinline__ fpair slab_shfl(fpair a, int src) {
   return fpair(__shfl_sync(0xffffffffu, a.v.x, src), __shfl_sync(0xffffffffu, a.v.y, src));
 }
 
-// 225^3, 9 components: 0.311 -> 0.275 ms a launch (the 3-field operator 428 -> 390 us) against one
-// pencil a lane group: 259 M -> 126 M warp instructions. It is bound by shared-memory
-// accesses now (72 % of the L1 data pipe; FP32 pipe 45 %, issue 39 %): a pencil passes through
-// shared memory once between its two register DFTs, and once between the y and x passes.
+// 225^3, 9 components: 0.311 -> 0.270 ms a launch (the 3-field operator 428 -> 383 us) against one
+// pencil a lane group: 248 M -> 123 M warp instructions. Shared-memory accesses weigh most
+// (71 % of the L1 data pipe; FP32 pipe 42 %, issue 37 %): a pencil passes through
+// shared memory once between its two register DFTs, and once between the y and x passes. 128
+// registers a thread (15 warps, one CTA an SM) leave 92 bytes of spills.
 template <int R, bool ZB, int NT = kSlabMaxThreads>
 __global__ void __launch_bounds__(NT) k_slab(SlabArgs a) {
   using F = fpair;
