@@ -2179,8 +2179,9 @@ hom_status hom_bounds_batched(hom_ctx* ctx, int32_t n, const hom_problem* probs,
   //   23: 128 9.1 / 8.5 / 7.2* / 7.3;  256 11.2 / 10.8 / 10.5* / 12.4;  512 16.3 / 15.7* / 17.7 / 22.1;  2048 50* / 56 / 65 / 107
   //   41: 256 28.1 / 21.7 / 20.9* / 22.3;  512 33.1 / 27.5* / 28.8 / 35.7;  2048 84.7* / 87.6 / 101 / 131
   //   63: 64 31.6 / 18.6 / 11.6 / 8.0*;  512 52.2 / 37.4 / 34.9* / 37.6;  2048 132* / 117 / 119 / 138
-  //   113: 256 87 / 53 / 41 / 35*;  2048 250 / 216* / 208 / 220
-  // and FP64 23: 512 53.9 / 45.2 / 51.2* / 105;  2048 130* / 145 / 182 / 283;  63: 1024 581 / 464 / 395* / 403.
+  //   89: 126 147 / 79 / 56 / 42*;  1024 266 / 203 / 220 / 204*
+  //   113: 256 87 / 53 / 41 / 35*;  2048 250 / 216 / 208* / 220
+  // and FP64 23: 512 53.9 / 45.2* / 51.2 / 105;  1024 79.5* / 82.5 / 101 / 149;  63: 1024 581 / 464 / 395* / 403.
   // CTAs of 512 threads (15 clusters of 8 at once) where the longest task is a large part of a
   // cluster's share of the batch, else 256 (36 clusters): 64 cells of mixed N 235 ms with one CTA a task, 32
   // (512), 41 (256), FP64 452 and 493; 256 of them 266, 92 and 68, FP64 1016 and 780; 63 cells of N = 89 147, 47 and
@@ -2193,7 +2194,8 @@ hom_status hom_bounds_batched(hom_ctx* ctx, int32_t n, const hom_problem* probs,
       longest = std::max(longest, w);
     }
     int c = bp.Mmax <= 64 ? 4 : 8;
-    while (c > 1 && work * c > (f32 ? 24.0 : 48.0) * bp.Mmax * longest) c /= 2;
+    const double M = bp.Mmax, room = f32 ? std::max(24.0 * M, M * M / 4) : std::max(44.0 * M, M * M / 2);
+    while (c > 1 && work * c > room * longest) c /= 2;
     size_t sm_ = 0;
     const int clusters = grid_for(cap0, 256, c, &sm_, c > 1) / c;
     *cl = c;
